@@ -55,6 +55,7 @@ constexpr int kCtlRoute = 16;   // 0: route (a); nonzero: route (b)
 constexpr int kCtlM = 17;       // largest slot - asc * cap / n of a pair
 constexpr int kCtlCompact = 18; // route (b): compacted pairs
 constexpr int kCtlShift = 19;   // b of the pair keys
+constexpr int kCtlHome = 20;    // home slots of a table too big for the cache: 0 by the minimum, 1 by both labels
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
     // 64-bit finaliser of MurmurHash3
@@ -94,33 +95,60 @@ __global__ void k_ms_prepare(const int32_t* __restrict__ asc, const int32_t* __r
     }
 }
 
-__global__ void k_ms_setcap(uint32_t* ctl, int64_t n, int64_t cap_max, int sh, int force_sort) {
+// Table capacity: a power of two that holds twice the bound on the distinct
+// pairs while that stays within n, else the bound itself (there are at most
+// n pairs; white noise fills a table of n slots to about a third).
+__device__ __forceinline__ unsigned long long table_capacity(const uint32_t* ctl, int64_t n, int64_t cap_max) {
     const unsigned long long pairs = (unsigned long long)ctl[0] * ctl[1];
     const unsigned long long bound = pairs < (unsigned long long)n ? pairs : (unsigned long long)n;
-    // twice the bound on the distinct pairs while that stays within n, else
-    // the bound itself (there are at most n pairs; white noise fills a
-    // table of n slots to about a third)
     const unsigned long long want = 2 * bound <= (unsigned long long)n ? 2 * bound : bound;
     unsigned long long cap = 64;
     while (cap < want) cap <<= 1;
-    if ((long long)cap > cap_max) cap = (unsigned long long)cap_max;
-    ctl[2] = (uint32_t)cap;  // cap_max <= 2^31
-    ctl[3] = 0;
-    // home-slot multiplier: asc * cap / n as (asc * F) >> 32, F = cap * 2^32 / n
-    const unsigned long long f = (cap << 32) / (unsigned long long)n;
-    ctl[9] = (uint32_t)f;
-    ctl[10] = (uint32_t)(f >> 32);
-    ctl[kCtlRoute] = (cap <= kCacheResidentSlots || force_sort) ? 1u : 0u;
-    ctl[kCtlM] = 0;
-    ctl[kCtlCompact] = 0;
-    ctl[kCtlShift] = (uint32_t)sh;
+    return (long long)cap > cap_max ? (unsigned long long)cap_max : cap;
 }
 
-__global__ void k_ms_clear(unsigned long long* keys, const uint32_t* ctl) {
-    const int64_t slots = (int64_t)ctl[2] + kPad;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots;
-         i += (int64_t)gridDim.x * blockDim.x)
-        keys[i] = kEmpty;
+constexpr int kHubSamples = 1 << 14;
+constexpr int kHubCounters = 1 << 14;  // in table_vals, which nothing else uses before the ranks
+constexpr uint32_t kHubVotes = 24;
+
+// Empties the table and the vote counters and writes the control words
+// (every block works the capacity out for itself: one launch fewer).
+__global__ void __launch_bounds__(kThreads) k_ms_clear(unsigned long long* keys, uint32_t* votes, uint32_t* ctl,
+                                                       int64_t n, int64_t cap_max, int sh, int force_sort) {
+    const unsigned long long cap = table_capacity(ctl, n, cap_max);
+    const int64_t slots = (int64_t)cap + kPad, t0 = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (t0 == 0) {
+        ctl[2] = (uint32_t)cap;  // cap_max <= 2^31
+        ctl[3] = 0;
+        // home-slot multiplier: asc * cap / n as (asc * F) >> 32, F = cap * 2^32 / n
+        const unsigned long long f = (cap << 32) / (unsigned long long)n;
+        ctl[9] = (uint32_t)f;
+        ctl[10] = (uint32_t)(f >> 32);
+        ctl[kCtlRoute] = (cap <= kCacheResidentSlots || force_sort) ? 1u : 0u;
+        ctl[kCtlHome] = force_sort ? 1u : 0u;
+        ctl[kCtlM] = 0;
+        ctl[kCtlCompact] = 0;
+        ctl[kCtlShift] = (uint32_t)sh;
+    }
+    for (int64_t i = t0; i < slots; i += (int64_t)gridDim.x * kThreads) keys[i] = kEmpty;
+    if (cap > kCacheResidentSlots && t0 < kHubCounters) votes[t0] = 0;
+}
+
+// The home-slot rule of a table too big for the cache.  Homes by the
+// minimum (route (a)) give the pairs of one minimum one window of kSpread
+// slots, which is right while every minimum meets few maxima.  A minimum whose
+// basin touches thousands of maxima (a deep valley in a noisy plain) turns
+// that window into one long cluster: 11.3 ms of insert for 16.7M vertices of
+// eight Gaussians plus noise, against 0.1 ms with homes by both labels.  So
+// kHubSamples vertices vote with their minima, and a minimum holding
+// kHubVotes of them (0.15 % of the vertices; a counter gets one vote on
+// average otherwise) selects homes by both labels and route (b).
+__global__ void __launch_bounds__(kThreads) k_ms_vote(const int32_t* __restrict__ asc, int64_t n, uint32_t* votes,
+                                                      uint32_t* ctl) {
+    if (ctl[2] <= kCacheResidentSlots) return;
+    const int t = blockIdx.x * kThreads + threadIdx.x;
+    const uint32_t a = (uint32_t)asc[(int64_t)t * n / kHubSamples];
+    if (atomicAdd(&votes[(a * 0x9E3779B1u) >> 18], 1u) + 1 == kHubVotes) ctl[kCtlRoute] = ctl[kCtlHome] = 1u;
 }
 
 // asc * cap / n by a fixed-point multiply (f = cap * 2^32 / n), no division.
@@ -132,11 +160,16 @@ __device__ __forceinline__ uint32_t slot_base(uint32_t asc, unsigned long long f
 // its minimum's id plus a small random spread.  The minimum of a vertex
 // lies near the vertex, so the vertices of a warp, and the warps in flight,
 // probe a narrow band of the table (L2 hits instead of random DRAM
-// sectors), and a pair's slot is at most M past asc * cap / n.
-__device__ __forceinline__ uint32_t home_slot(uint32_t asc, unsigned long long key, uint32_t cap,
-                                              unsigned long long f) {
+// sectors), and a pair's slot is at most M past asc * cap / n.  With
+// `both`, proportional to the mean of its two extrema's ids instead: as
+// near to the vertex where both extrema are, and the many pairs of one
+// far-reaching extremum spread out with their other ends.
+__device__ __forceinline__ uint32_t home_slot(uint32_t asc, uint32_t desc, unsigned long long key, uint32_t cap,
+                                              unsigned long long f, bool both) {
     if (cap <= kCacheResidentSlots) return (uint32_t)mix64(key) & (cap - 1);  // fits in cache: spread
-    return slot_base(asc, f) + (uint32_t)(mix64(key) & (kSpread - 1));
+    // a base is below cap for labels in [0, n); labels outside (already
+    // reported) must not leave the table either
+    return min(slot_base(both ? (asc + desc) >> 1 : asc, f), cap) + (uint32_t)(mix64(key) & (kSpread - 1));
 }
 
 // Linear probing over the cap + kPad slots; `fresh` when this call stored
@@ -219,8 +252,12 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
     const uint32_t cap = ctl[2];
     const uint32_t lim = cap + kPad;
     const int sh = (int)ctl[kCtlShift];
-    const bool ordered = ctl[kCtlRoute] == 0u;
+    // fixed before this kernel starts (ctl[kCtlRoute] changes while it runs):
+    // every insert of a key has to follow the same probes
+    const bool both = ctl[kCtlHome] != 0u;
+    const bool ordered = cap > kCacheResidentSlots && !both;
     const unsigned long long f = (unsigned long long)ctl[9] | ((unsigned long long)ctl[10] << 32);
+    const uint32_t dmask = (1u << sh) - 1u;  // sh = ceil(log2 n) <= 31
     const int lane = threadIdx.x & 31;
     constexpr int64_t kStep = (int64_t)kThreads * kInsJ;
     uint32_t added = 0, far = 0;
@@ -250,7 +287,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
         for (int j = 0; j < kInsJ; ++j) {
             slot[j] = 0;
             if (probing >> j & 1u) {
-                h[j] = home_slot(a[j], key[j], cap, f);
+                h[j] = home_slot(a[j], (uint32_t)key[j] & dmask, key[j], cap, f, both);
                 w[j] = keys[h[j]];
             }
         }
@@ -657,13 +694,15 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
     }
     MSC_LAUNCHED();
     {
-        TraceScope ts_("msid.setcap", s);
-        k_ms_setcap<<<1, 1, 0, s>>>(sc.ctl, n, sc.cap_max, sh, sorted_keys ? 1 : 0);
+        TraceScope ts_("msid.clear", s);
+        // at least kHubCounters threads, so that every vote counter is cleared
+        const int grid = std::max(grid_for(sc.cap_max + kPad, 4), kHubCounters / kThreads);
+        k_ms_clear<<<grid, kThreads, 0, s>>>(sc.table_keys, sc.table_vals, sc.ctl, n, sc.cap_max, sh, sorted_keys ? 1 : 0);
     }
     MSC_LAUNCHED();
-    {
-        TraceScope ts_("msid.clear", s);
-        k_ms_clear<<<grid_for(sc.cap_max + kPad, 4), kThreads, 0, s>>>(sc.table_keys, sc.ctl);
+    if (sc.cap_max > (int64_t)kCacheResidentSlots && !sorted_keys) {
+        TraceScope ts_("msid.vote", s);
+        k_ms_vote<<<kHubSamples / kThreads, kThreads, 0, s>>>(asc, n, sc.table_vals, sc.ctl);
     }
     MSC_LAUNCHED();
     {
