@@ -47,6 +47,39 @@ __device__ __forceinline__ int32_t ld_volatile_s32(const int32_t* p) {
     return v;
 }
 
+// A block's walk over the tiles first, first + step, first + 2 step, ... of
+// a tx x ty x .. grid of tiles (x fastest; counts fit 32 bits, as every tile
+// holds a vertex): the coordinates advance by the step's own, so a tile
+// costs a few additions instead of two divisions.
+struct TileWalk {
+    int32_t tx, ty;
+    int32_t x, y, z;     // the current tile
+    int32_t sx, sy, sz;  // the step
+    __device__ __forceinline__ TileWalk(int32_t tx_, int32_t ty_, uint32_t first, uint32_t step) : tx(tx_), ty(ty_) {
+        split(first, x, y, z);
+        split(step, sx, sy, sz);
+    }
+    __device__ __forceinline__ void split(uint32_t t, int32_t& a, int32_t& b, int32_t& c) const {
+        const uint32_t q = t / (uint32_t)tx;
+        a = (int32_t)(t - q * (uint32_t)tx);
+        c = (int32_t)(q / (uint32_t)ty);
+        b = (int32_t)(q - (uint32_t)c * (uint32_t)ty);
+    }
+    __device__ __forceinline__ void advance() {
+        x += sx;
+        y += sy;
+        z += sz;
+        if (x >= tx) {
+            x -= tx;
+            ++y;
+        }
+        if (y >= ty) {
+            y -= ty;
+            ++z;
+        }
+    }
+};
+
 // ----------------------------------------------------------------------------
 // host side
 struct Device {

@@ -261,9 +261,7 @@ int msc_cc_mask(const uint8_t* mask, msc_grid g, int32_t conn, int32_t* label, v
     (void)ws;
     if (!grid_ok(g) || !mask || !label || !d_status || (conn != 6 && conn != 14)) return MSC_ERR_ARG;
     if (ws_bytes < msc_workspace_bytes(MSC_OP_CC_MASK, grid_n(g), 0)) return MSC_ERR_WS;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    MSC_TRY(cudaMemsetAsync(d_status, 0, sizeof(int32_t), s));
-    return run_cc_mask(mask, g, conn, label, d_status, s);
+    return run_cc_mask(mask, g, conn, label, d_status, static_cast<cudaStream_t>(stream));  // sets *d_status first
 }
 
 int msc_cc_mesh(const int32_t* row, const int32_t* col, int32_t n, int32_t* label, void* ws, size_t ws_bytes,

@@ -73,3 +73,52 @@ def test_ms_id_reports_labels_outside_a_large_table(m, bad):
     with pytest.raises(m.MSCError) as e:
         m.ms_id(cuda(asc), cuda(desc))
     assert e.value.code == m.ERR_ARG
+
+
+# ---------------------------------------------------------------------------
+# mask components: contacts across tile faces, mask rows of every alignment
+
+
+@pytest.mark.parametrize("conn", [6, 14])
+@pytest.mark.parametrize("dims", [(64, 8, 8), (65, 9, 9), (129, 17, 25), (63, 16, 8), (200, 31, 33), (130, 7, 41)])
+@pytest.mark.parametrize("density", [0.02, 0.25, 0.5, 0.9, 1.0])
+def test_cc_mask_tile_contacts(m, oracle_mod, conn, dims, density):
+    n = dims[0] * dims[1] * dims[2]
+    mask = (np.random.default_rng(n).random(n) < density).astype(np.uint8) * 255
+    np.testing.assert_array_equal(host(m.cc_mask(cuda(mask), dims, conn)), oracle_mod.cc_grid(mask, dims, conn))
+
+
+@pytest.mark.parametrize("conn", [6, 14])
+@pytest.mark.parametrize("offset", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("nx", [61, 64, 66, 72])
+def test_cc_mask_unaligned_mask(m, oracle_mod, conn, offset, nx):
+    dims = (nx, 18, 11)
+    n = dims[0] * dims[1] * dims[2]
+    mask = (np.random.default_rng(nx + offset).random(n) < 0.35).astype(np.uint8)
+    buf = torch.empty(n + offset, dtype=torch.uint8, device="cuda")  # the mask ends where its buffer ends
+    buf[offset:] = cuda(mask)
+    np.testing.assert_array_equal(host(m.cc_mask(buf[offset:], dims, conn)), oracle_mod.cc_grid(mask, dims, conn))
+
+
+@pytest.mark.parametrize("conn", [6, 14])
+def test_cc_mask_single_contacts(m, oracle_mod, conn):
+    """Pairs of voxels joined by one edge only, across every side and diagonal of a tile."""
+    dims = (128, 16, 16)
+    offs = [(1, 0, 0), (0, 1, 0), (0, 0, 1), (1, 1, 0), (1, 0, 1), (0, 1, 1), (1, 1, 1), (-1, 1, 0), (1, -1, 0)]
+    ends = [(63, 7, 7), (63, 3, 4), (20, 7, 3), (20, 3, 7), (30, 7, 7), (63, 7, 2), (63, 2, 7), (64, 7, 7), (10, 2, 2)]
+    for x, y, z in ends:
+        for dx, dy, dz in offs:
+            mask = np.zeros((dims[2], dims[1], dims[0]), np.uint8)
+            mask[z, y, x] = mask[z + dz, y + dy, x + dx] = 1
+            got = host(m.cc_mask(cuda(mask.ravel()), dims, conn))
+            np.testing.assert_array_equal(got, oracle_mod.cc_grid(mask.ravel(), dims, conn))
+
+
+def test_cc_mask_more_contacts_than_the_queue(m, oracle_mod):
+    """Isolated voxels on both sides of the faces: hundreds of contacts in one tile."""
+    dims = (128, 16, 16)
+    z, y, x = np.meshgrid(*(np.arange(d) for d in reversed(dims)), indexing="ij")
+    mask = ((x + y) % 2 == 0) & ((z == 7) | (z == 8)) | ((x + z) % 2 == 0) & ((y == 7) | (y == 8))
+    mask = mask.astype(np.uint8).ravel()
+    for conn in (6, 14):
+        np.testing.assert_array_equal(host(m.cc_mask(cuda(mask), dims, conn)), oracle_mod.cc_grid(mask, dims, conn))
