@@ -81,11 +81,18 @@ __device__ __forceinline__ void union_s(int* L, int a, int b) {
 // write is an atomicMin: labels only ever decrease (every entry points at a
 // smaller or equal id of the same component), so a halving write can never
 // undo a hook or overwrite a final root written by another thread.
+// Cached reads: once most vertices share a root, nearly every find ends at
+// its word, and reads that all go to one L2 slice serialise (mesh of 256^3
+// vertices: 1.36 ms for uniting the second neighbours, 0.37 with the L1
+// serving them).  A
+// stale read is an older ancestor of the same component; a union that took
+// it for a root learns the present value from its atomicMin and goes on from
+// there.
 __device__ __forceinline__ int32_t find_g(int32_t* L, int32_t x) {
     for (uint32_t it = 0; it < kUnionLimit; ++it) {
-        const int32_t p = ld_volatile_s32(L + x);
+        const int32_t p = ld_cached_s32(L + x);
         if (p == x) return x;
-        const int32_t gp = ld_volatile_s32(L + p);
+        const int32_t gp = ld_cached_s32(L + p);
         if (gp != p) atomicMin(L + x, gp);
         x = gp;
     }
@@ -104,7 +111,7 @@ __device__ __forceinline__ void union_g(int32_t* L, int32_t a, int32_t b, int32_
         }
         const int32_t old = atomicMin(L + b, a);
         if (old == b) return;
-        b = old;
+        b = old;  // below b, fresh from L2
     }
     record_error(status, MSC_ERR_INTERNAL);
 }
@@ -601,15 +608,21 @@ __global__ void __launch_bounds__(kFlatThreads) k_flatten(int32_t* label, int64_
 // mesh
 
 // Mesh kernels (subgraph sampling, after the Afforest scheme):
-//   1. label[v] = v; unite every vertex with its first and second neighbour
-//      (one lane per vertex and round);
-//   2. flatten; sample 1024 vertices and take the most frequent label --
+//   1. label[v] = v;
+//   2. every vertex unites its first two neighbours, both read at once: any
+//      read of a row's start fetches a good part of the row from DRAM (64
+//      bytes at a time), so one launch per neighbour read the columns twice
+//      (256^3 vertices, 13.7 columns each: 1.59 ms as two launches with
+//      uncached finds, 0.54 with a plain hook to the first neighbour as a
+//      pass of its own and cached finds, 0.38 as one launch; reading every
+//      column once takes 0.14);
+//   3. flatten; sample 1024 vertices and take the most frequent label --
 //      on a well-connected mesh, nearly every vertex is already in that
 //      component;
-//   3. every vertex outside it unites all its remaining edges (8 lanes per
+//   4. every vertex outside it unites all its remaining edges (8 lanes per
 //      row); an edge to a vertex of the frequent component is found from
 //      this side, since the adjacency is symmetric;
-//   4. flatten.
+//   5. flatten.
 // Every union hooks the larger root under the smaller, so the final root of
 // a component is its smallest vertex id, whatever the order of unions.
 constexpr int kRowLanes = 8;
@@ -620,18 +633,17 @@ __global__ void k_mesh_init(int32_t* label, int32_t n) {
         label[v] = (int32_t)v;
 }
 
-// Unite every vertex with its k-th neighbour (k = 0 or 1).
-__global__ void k_mesh_link_k(const int32_t* __restrict__ row, const int32_t* __restrict__ col, int32_t n,
-                              int k, int32_t* label, int32_t* status) {
+__global__ void __launch_bounds__(256) k_mesh_link(const int32_t* __restrict__ row, const int32_t* __restrict__ col,
+                                                   int32_t n, int32_t* label, int32_t* status) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t e = row[v] + k;
-        if (e >= row[v + 1]) continue;
-        const int32_t u = col[e];
-        if ((uint32_t)u >= (uint32_t)n) {
+        const int32_t e = row[v], e1 = row[v + 1];
+        const int32_t u0 = e < e1 ? col[e] : (int32_t)v, u1 = e + 1 < e1 ? col[e + 1] : (int32_t)v;
+        if ((uint32_t)u0 >= (uint32_t)n || (uint32_t)u1 >= (uint32_t)n) {
             record_error(status, MSC_ERR_ARG);
             continue;
         }
-        union_g(label, (int32_t)v, u, status);
+        if (u0 != v) union_g(label, (int32_t)v, u0, status);
+        if (u1 != v) union_g(label, (int32_t)v, u1, status);
     }
 }
 
@@ -657,21 +669,21 @@ __global__ void __launch_bounds__(kSamples) k_mesh_sample(const int32_t* label, 
             }
             __syncthreads();
         }
-    if (t == 0) {
-        int32_t best = s[0], best_len = 0, cur = s[0], len = 0;
-        for (int i = 0; i < kSamples; ++i) {
-            if (s[i] == cur) ++len;
-            else {
-                cur = s[i];
-                len = 1;
-            }
-            if (len > best_len) {
-                best_len = len;
-                best = cur;
-            }
+    // each run's first entry finds its end; (length, smallest label) wins
+    __shared__ unsigned long long best;
+    if (t == 0) best = 0;
+    __syncthreads();
+    if (t == 0 || s[t - 1] != s[t]) {
+        int lo = t + 1, hi = kSamples;  // first entry past the run
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (s[mid] == s[t]) lo = mid + 1;
+            else hi = mid;
         }
-        *frequent = best;
+        atomicMax(&best, (unsigned long long)(lo - t) << 32 | (uint32_t)~s[t]);
     }
+    __syncthreads();
+    if (t == 0) *frequent = (int32_t)~(uint32_t)best;
 }
 
 // Vertices outside the frequent component unite their remaining edges.
@@ -682,19 +694,25 @@ __global__ void __launch_bounds__(256) k_mesh_hook(const int32_t* __restrict__ r
     const int lane = threadIdx.x & 31, sub = lane & (kRowLanes - 1);
     const int32_t big = *frequent;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) / 32;
-    constexpr int kPerWarp = 32 / kRowLanes;
-    for (int64_t wbase = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32) * kPerWarp; wbase < n;
-         wbase += warps * kPerWarp) {
-        const int64_t v = wbase + lane / kRowLanes;
-        if (v >= n || label[v] == big) continue;
-        const int32_t e1 = row[v + 1];
-        for (int32_t e = row[v] + 2 + sub; e < e1; e += kRowLanes) {
-            const int32_t u = col[e];
-            if ((uint32_t)u >= (uint32_t)n) {
-                record_error(status, MSC_ERR_ARG);
-                continue;
+    for (int64_t wbase = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32) * 32; wbase < n; wbase += warps * 32) {
+        // 32 vertices' labels at once, then the rows that are wanted, four at a time
+        const int64_t own = wbase + lane;
+        const uint32_t want = __ballot_sync(0xffffffffu, own < n && label[own] != big);
+        if (!want) continue;
+#pragma unroll 1
+        for (int i = 0; i < kRowLanes; ++i) {
+            const int q = (32 / kRowLanes) * i + lane / kRowLanes;
+            if (!(want >> q & 1u)) continue;
+            const int64_t v = wbase + q;
+            const int32_t e1 = row[v + 1];
+            for (int32_t e = row[v] + 2 + sub; e < e1; e += kRowLanes) {
+                const int32_t u = col[e];
+                if ((uint32_t)u >= (uint32_t)n) {
+                    record_error(status, MSC_ERR_ARG);
+                    continue;
+                }
+                union_g(label, (int32_t)v, u, status);
             }
-            union_g(label, (int32_t)v, u, status);
         }
     }
 }
@@ -753,9 +771,9 @@ int run_cc_mesh(const int32_t* row, const int32_t* col, int32_t n, int32_t* labe
         k_mesh_init<<<grid, 256, 0, s>>>(label, n);
     }
     MSC_LAUNCHED();
-    for (int k = 0; k < 2; ++k) {
+    {
         TraceScope ts_("mesh.link", s);
-        k_mesh_link_k<<<grid, 256, 0, s>>>(row, col, n, k, label, status);
+        k_mesh_link<<<grid, 256, 0, s>>>(row, col, n, label, status);
     }
     MSC_LAUNCHED();
     {

@@ -122,3 +122,22 @@ def test_cc_mask_more_contacts_than_the_queue(m, oracle_mod):
     mask = mask.astype(np.uint8).ravel()
     for conn in (6, 14):
         np.testing.assert_array_equal(host(m.cc_mask(cuda(mask), dims, conn)), oracle_mod.cc_grid(mask, dims, conn))
+
+
+# ---------------------------------------------------------------------------
+# mesh components: rows of any order, vertices with no, one or two neighbours
+
+
+@pytest.mark.parametrize("n,edges", [(1, 0), (2, 1), (33, 20), (5000, 1500), (70001, 60000), (70001, 200000)])
+@pytest.mark.parametrize("rows", ["ascending", "descending", "shuffled"])
+def test_cc_mesh_row_orders(m, oracle_mod, n, edges, rows):
+    rng = np.random.default_rng(n + edges)
+    a, b = rng.integers(0, n, edges), rng.integers(0, n, edges)
+    a, b = a[a != b], b[a != b]
+    src, dst = np.concatenate([a, b]), np.concatenate([b, a])
+    key = {"ascending": dst, "descending": -dst, "shuffled": rng.random(dst.size)}[rows]
+    at = np.lexsort((key, src))
+    row = np.zeros(n + 1, np.int32)
+    row[1:] = np.cumsum(np.bincount(src, minlength=n))
+    col = dst[at].astype(np.int32)
+    np.testing.assert_array_equal(host(m.cc_mesh(cuda(row), cuda(col))), oracle_mod.cc_csr(row, col))
