@@ -140,7 +140,7 @@ MSC_API int msc_compress(int32_t* ptr, int32_t n, void* ws, size_t ws_bytes, int
  * msc_compress does, with the same arguments minus the workspace, and
  * allocates nothing (no cudaMalloc, cudaFree or allocating library
  * routine).  It is an ordinary host call that enqueues work on `stream`
- * (a memset, an occupancy query and about log5(n) + 3 kernel launches), so
+ * (a memset, occupancy queries and up to five kernel launches), so
  * it must not be made from a host function enqueued on a stream, where CUDA
  * calls are not allowed.
  *   n  at most MSC_NOALLOC_MAX_N; larger n returns MSC_ERR_TOO_LARGE.

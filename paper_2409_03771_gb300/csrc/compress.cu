@@ -4,11 +4,12 @@
 // d[u] may already see this sweep's write, which only lengthens the jump.
 //
 // GPU form: one launch per sweep over all vertices (eight vertices per
-// thread, lane-consecutive).  Each vertex follows up to kHops (4) hops per
+// thread, lane-consecutive), the late sweeps together in one cooperative
+// launch.  Each vertex follows up to kHops (4) hops per
 // sweep (d[v] <- d[d[d[d[d[v]]]]]), so a sweep at least quintuples every
 // pointer's reach for the same 8 bytes of pointer read and write per
-// vertex; the extra reads mostly hit the cache.  Launched ceil(log5 n) + 2
-// times.  Each sweep counts the vertices it changed; a sweep whose
+// vertex; the extra reads mostly hit the cache.  At most ceil(log5 n) + 2
+// sweeps.  Each sweep counts the vertices it changed; a sweep whose
 // predecessor changed nothing returns at once, so no host synchronisation
 // is needed.  A sweep also appends the vertices it changed to an active
 // list (block-aggregated atomics) once the previous sweep's count is at
@@ -26,6 +27,7 @@
 #include <mutex>
 
 #include "compress.cuh"
+#include "coop.cuh"
 
 namespace msc {
 namespace {
@@ -107,16 +109,18 @@ __device__ __forceinline__ uint32_t jump_group(const int32_t* p, int32_t n, cons
     return moved;
 }
 
+// One sweep over array `which`, by the blocks of gridDim.x.  Returns the
+// vertices the previous sweep changed; with 0 there is nothing to do.
 template <bool CHECKED>
-__global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, uint32_t build_max,
-                                                   int32_t* status) {
-    const JumpArray A = blockIdx.y ? pr.a[1] : pr.a[0];
+__device__ __forceinline__ uint32_t jump_sweep(const JumpPair& pr, int which, int step, uint32_t build_max,
+                                               int32_t* status) {
+    const JumpArray A = which ? pr.a[1] : pr.a[0];
     const int32_t n = pr.n;
     int32_t* p = A.p;
-    const uint32_t prev = step == 0 ? (uint32_t)n : A.ctl->cnt[step - 1];
-    if (prev == 0) return;
+    const uint32_t prev = step == 0 ? (uint32_t)n : __ldcg(&A.ctl->cnt[step - 1]);
+    if (prev == 0) return 0;
     // the previous sweep's list is complete only if its changes fitted
-    const bool from_list = step > 0 && A.ctl->built[step - 1] != 0 && (int64_t)prev <= A.list_cap;
+    const bool from_list = step > 0 && __ldcg(&A.ctl->built[step - 1]) != 0 && (int64_t)prev <= A.list_cap;
     const bool build = prev <= build_max;
     if (build && blockIdx.x == 0 && threadIdx.x == 0) A.ctl->built[step] = 1u;
     int32_t* out_list = (step & 1) ? A.list1 : A.list0;
@@ -209,14 +213,44 @@ __global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, 
     if (step == 0 && pr.roots) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) roots_seen += __shfl_xor_sync(0xffffffffu, roots_seen, o);
-        if (lane == 0 && roots_seen) atomicAdd(&pr.roots[blockIdx.y], roots_seen);
+        if (lane == 0 && roots_seen) atomicAdd(&pr.roots[which], roots_seen);
     }
+    return prev;
 }
 
-__global__ void k_jump_finish(const JumpPair pr, int count, int last, int32_t* status) {
-    for (int i = 0; i < count; ++i)
-        if (pr.a[i].ctl->cnt[last] != 0u) record_error(status, MSC_ERR_NOT_CONVERGED);
+template <bool CHECKED>
+__global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, uint32_t build_max, int32_t* status) {
+    jump_sweep<CHECKED>(pr, blockIdx.y, step, build_max, status);
 }
+
+// The sweeps from `first` on, in one cooperative launch with a grid barrier
+// between two of them, until nothing moves or the last possible sweep: the
+// later sweeps have little or nothing left to do (paths of more than 5^k
+// steps), and a launch for each was most of what they cost.
+template <bool CHECKED>
+__global__ void __launch_bounds__(kThreads) k_jump_tail(const JumpPair pr, int count, int first, int steps,
+                                                        uint32_t build_max, uint32_t* barrier, int32_t* status) {
+    GridBarrier bar{barrier, gridDim.x, 0};
+    for (int step = first; step < steps; ++step) {
+        uint32_t prev = 0;
+        for (int i = 0; i < count; ++i) prev |= jump_sweep<CHECKED>(pr, i, step, build_max, status);
+        if (prev == 0) return;  // the same in every block: read before this step's writes
+        if (!grid_barrier(bar, status)) return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        for (int i = 0; i < count; ++i)
+            if (__ldcg(&pr.a[i].ctl->cnt[steps - 1]) != 0u) record_error(status, MSC_ERR_NOT_CONVERGED);
+}
+
+// Sweeps launched over the whole GPU before the tail: the ones that usually
+// have work.  All sweeps of a small array go into the tail (64^3 vertices:
+// 62 us as eleven launches, 28 as one; 256^3, four launches and the tail: 163
+// -> 127).  Large arrays keep eight launches, so that only paths of more than
+// 390 000 steps meet the tail's smaller grid.
+constexpr int64_t kTailVertices = 1 << 20;
+constexpr int64_t kLargeVertices = 1 << 24;
+int full_sweeps(int64_t n) { return n <= kTailVertices ? 0 : n < kLargeVertices ? 4 : 8; }
+constexpr int kTailBlocksPerSm = 2;  // leaves room to start beside other streams' kernels
 
 }  // namespace
 
@@ -261,24 +295,28 @@ int run_compress(int32_t* const* ptrs, int count, int32_t n, const CompressScrat
     const int64_t fill_max = std::min<int64_t>(sc.list_cap + sc.list_cap / 2, UINT32_MAX);
     const uint32_t build_max = tune.fill_lists ? (uint32_t)fill_max : ((uint32_t)n >> build_shift);
     auto kern = tune.trusted ? k_jump<false> : k_jump<true>;
-    int occ = 1;
-    MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0));
     const int64_t chunks = ceil_div(n, kChunkV);
-    const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, (int64_t)current_device().sms * std::max(occ, 1)));
     const int steps = compress_steps(n);
-    for (int st = 0; st < steps; ++st) {
-        {
-            TraceScope ts_("compress.jump", s);
-            kern<<<dim3(gx, count), kThreads, 0, s>>>(pr, st, build_max, status);
+    const int full = std::min(full_sweeps(n), steps);
+    if (full > 0) {
+        int occ = 1;
+        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0));
+        const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, (int64_t)current_device().sms * std::max(occ, 1)));
+        for (int st = 0; st < full; ++st) {
+            {
+                TraceScope ts_("compress.jump", s);
+                kern<<<dim3(gx, count), kThreads, 0, s>>>(pr, st, build_max, status);
+            }
+            MSC_LAUNCHED();
         }
-        MSC_LAUNCHED();
     }
-    {
-        TraceScope ts_("compress.finish", s);
-        k_jump_finish<<<1, 1, 0, s>>>(pr, count, steps - 1, status);
-    }
-    MSC_LAUNCHED();
-    return MSC_OK;
+    auto tail = tune.trusted ? k_jump_tail<false> : k_jump_tail<true>;
+    int blocks = 0;
+    const int r = coop_blocks(
+        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * kTailBlocksPerSm), &blocks);
+    if (r) return r;
+    TraceScope ts_("compress.tail", s);
+    return coop_launch(tail, blocks, kThreads, 0, s, pr, count, full, steps, build_max, &sc.ctl[0].barrier, status);
 }
 
 }  // namespace msc

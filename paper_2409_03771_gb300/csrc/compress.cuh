@@ -12,6 +12,8 @@ constexpr int kMaxJumpSteps = 64;
 struct JumpCtl {
     uint32_t cnt[kMaxJumpSteps];    // vertices changed in each step
     uint32_t built[kMaxJumpSteps];  // step wrote its changed vertices to a list
+    uint32_t barrier;               // array 0: the tail's grid barrier
+    uint32_t pad[31];
 };
 
 struct CompressTune {
@@ -22,7 +24,7 @@ struct CompressTune {
     uint32_t* roots = nullptr;  // roots[i] += #self-pointers of array i (first sweep)
 };
 
-// Sweeps launched for n vertices: ceil(log5 n) + 2 (enough for any forest
+// Sweeps at most for n vertices: ceil(log5 n) + 2 (enough for any forest
 // at a fivefold advance per sweep; more are needed only by a cycle).
 int compress_steps(int64_t n);
 
