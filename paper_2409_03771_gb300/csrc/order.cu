@@ -26,12 +26,15 @@
 //               completed in L2 before they are written back.
 // The last pass files (vertex id, position) pairs into buckets of
 // consecutive ids instead of writing sorted keys, and the order field is
-// their inverse permutation (k_pair_split / k_pair_scatter_local).
+// their inverse permutation (k_pair_split / k_pair_scatter_local); while the
+// order array fits the L2 it scatters the positions itself.  Small fields go
+// through all four passes in one cooperative launch (k_ord_coop).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <type_traits>
 
+#include "coop.cuh"
 #include "radix.cuh"
 #include "sort.cuh"
 #include "tma.cuh"
@@ -190,6 +193,14 @@ __global__ void __launch_bounds__(kT) k_ord_scan(uint32_t* __restrict__ cnt, con
     }
 }
 
+// What a downsweep writes: the sorted (key, id) arrays, (id, position) pairs
+// filed by id bucket, or order[id] = position.  Scattering the order
+// straight from the last pass is best while the order array stays in L2:
+// 2^24 vertices of white noise 684 -> 632 us, of 256 levels 668 -> 545; 2^25
+// vertices 1266 against 1527.
+enum { kOutSorted, kOutBuckets, kOutOrder };
+constexpr int64_t kOrderDirectMax = 1 << 24;
+
 struct DownArgs {
     const float* f;            // pass 0: the field (keys made from it, ids implicit)
     const uint32_t* keys_in;   // other passes
@@ -216,7 +227,7 @@ constexpr size_t kDownSmem = 2 * kBufWords * 4 + kW * kB * 2 + 2 * kB * 4 + 32 *
 // instruction, whose cost grows with the number of distinct digits in the
 // warp, or eight ballots, whose cost does not (digit_peers in radix.cuh).
 
-template <bool FROM_F, bool BUCKET, int SHIFT>
+template <bool FROM_F, int OUT, int SHIFT>
 __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     uint32_t* buf = reinterpret_cast<uint32_t*>(smem);                     // [2][kTile words | kTile words]
@@ -334,7 +345,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
             if (use_match) rank_tile(std::true_type{}, std::false_type{});
             else rank_tile(std::false_type{}, std::false_type{});
         }
-        if constexpr (BUCKET) s_bcnt[tid] = 0u;
+        if constexpr (OUT == kOutBuckets) s_bcnt[tid] = 0u;
         __syncthreads();
         {   // digit tid: warp counts -> tile-local start of each warp's run of
             // the digit (16-bit: at most kTile); output start of the tile's run
@@ -352,7 +363,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
             s_run[tid] = g + run;
         }
         __syncthreads();
-        if constexpr (!BUCKET) {
+        if constexpr (OUT == kOutSorted) {
             // values into registers first (the field pass makes them from the
             // index), so that bv is free for the staged keys
             uint32_t val[kI];
@@ -399,6 +410,19 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
                     }
                 }
             }
+        } else if constexpr (OUT == kOutOrder) {
+#pragma unroll
+            for (int k = 0; k < kI; ++k) {
+                const int li = wb + 32 * k;
+                if (li < cnt) {
+                    const uint32_t d = (dg[k / 4] >> (8 * (k & 3))) & 255u;
+                    const uint32_t pos = s_delta[d] + wh[d] + ((rk[k / 2] >> (16 * (k & 1))) & 0xffffu);
+                    const uint32_t id = bv[li];
+                    MSC_GUARD(id < (uint64_t)r.n && pos < (uint64_t)r.n, a.status, -146) a.vals_out[id] = (int32_t)pos;
+                }
+            }
+            __syncwarp();
+            for (int j = lane; j < kB / 2; j += 32) reinterpret_cast<uint32_t*>(wh)[j] = 0u;
         } else {
             // final positions straight from the ranks; (id, position) pairs
             // regrouped by id bucket, each bucket's run written with
@@ -462,24 +486,24 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     }
 }
 
-template <bool FROM_F, bool BUCKET, int SHIFT>
+template <bool FROM_F, int OUT, int SHIFT>
 int configure_down() {
     static int configured_dev = -1;  // the attribute is set once per device
     if (configured_dev != current_device().id) {
-        MSC_TRY(cudaFuncSetAttribute(k_ord_down<FROM_F, BUCKET, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        MSC_TRY(cudaFuncSetAttribute(k_ord_down<FROM_F, OUT, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kDownSmem));
         configured_dev = current_device().id;
     }
     return MSC_OK;
 }
 
-template <bool FROM_F, bool BUCKET, int SHIFT>
+template <bool FROM_F, int OUT, int SHIFT>
 int launch_down(const DownArgs& a, int blocks, cudaStream_t s, const char* label) {
-    const int rc = configure_down<FROM_F, BUCKET, SHIFT>();
+    const int rc = configure_down<FROM_F, OUT, SHIFT>();
     if (rc) return rc;
     {
         TraceScope ts_(label, s);
-        k_ord_down<FROM_F, BUCKET, SHIFT><<<blocks, kT, kDownSmem, s>>>(a);
+        k_ord_down<FROM_F, OUT, SHIFT><<<blocks, kT, kDownSmem, s>>>(a);
     }
     MSC_LAUNCHED();
     return MSC_OK;
@@ -503,11 +527,94 @@ int launch_up(const float* f, const uint32_t* keys, const Range& rg, int blocks,
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
+// The whole sort of a small field in one cooperative launch: the sort of
+// 2^18 vertices is 16 launches and fills otherwise (125 us, 93 replayed as a
+// graph, against 48 here; bound by the latency of the phases, some 10 us per
+// pass).  The data stays in L2 between the passes, so the last pass writes
+// order[id] = position straight away.  A digit that all keys share (the low
+// mantissa bits of small whole numbers) costs its count only.
+struct CoopOrderArgs {
+    const float* f;
+    uint32_t n;
+    int32_t* order;
+    uint32_t* key[2];
+    uint32_t* id[2];
+    uint32_t* scratch;  // kCoopScratchWords, then the barrier word
+    int32_t* status;
+};
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kCoopThreads) k_ord_coop(const CoopOrderArgs a) {
+    extern __shared__ __align__(16) uint8_t coop_smem[];
+    CoopSmem<uint32_t, ITEMS>& S = *reinterpret_cast<CoopSmem<uint32_t, ITEMS>*>(coop_smem);
+    GridBarrier bar{a.scratch + kCoopScratchWords, gridDim.x, 0};
+    int src = -1;  // the buffer holding the keys; -1: the field
+    bool nan = false;
+#pragma unroll 1
+    for (int p = 0; p < 4; ++p) {
+        const bool last = p == 3;
+        const uint32_t* kin = src < 0 ? nullptr : a.key[src];
+        const uint32_t* vin = src < 0 ? nullptr : a.id[src];
+        const int dst = src == 0;
+        const CoopPass r = coop_radix_pass<uint32_t, ITEMS>(
+            S, a.n, 8 * p, !last,
+            [&](uint32_t i) -> uint32_t {
+                if (kin) return kin[i];
+                const float x = a.f[i];
+                nan |= is_nan_bits(x);
+                return float_key(x);
+            },
+            [&](uint32_t i) -> uint32_t { return vin ? vin[i] : i; },
+            [&](uint32_t pos, uint32_t k, uint32_t id) {
+                if (last) {
+                    a.order[id] = (int32_t)pos;
+                } else {
+                    a.key[dst][pos] = k;
+                    a.id[dst][pos] = id;
+                }
+            },
+            a.scratch, bar, a.status);
+        if (r == kPassFailed) return;
+        if (r == kPassMoved) src = dst;
+    }
+    if (nan) record_error(a.status, MSC_ERR_NAN);
+}
+
+// Largest field sorted by k_ord_coop: with two tiles per block the passes
+// lose more by their double reading than the launches cost (2^21 vertices:
+// 135 us against 179 as launches; 3 * 10^6: 200 against 176).  Eight keys per
+// thread while that leaves one tile per block at two blocks per SM (262 144:
+// 48 us, 61 with sixteen; 10^6: 93 and 76).
+constexpr int64_t kOrderCoopMax = 1 << 21;
+static_assert(kCoopScratchWords + 1 <= kOrderCntWords, "the barrier word follows the counts");
+
+template <int ITEMS>
+int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
+    using Smem = CoopSmem<uint32_t, ITEMS>;
+    static int configured_dev = -1;
+    if (configured_dev != current_device().id) {
+        MSC_TRY(cudaFuncSetAttribute(k_ord_coop<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)));
+        configured_dev = current_device().id;
+    }
+    int blocks = 0;
+    const int r = coop_blocks(k_ord_coop<ITEMS>, kCoopThreads, sizeof(Smem),
+                              std::min<int64_t>(ceil_div(a.n, Smem::kTile), kCoopMaxBlocks), &blocks);
+    if (r) return r;
+    MSC_TRY(cudaMemsetAsync(a.scratch + kCoopScratchWords, 0, sizeof(uint32_t), s));
+    TraceScope ts_("order.coop", s);
+    return coop_launch(k_ord_coop<ITEMS>, blocks, kCoopThreads, sizeof(Smem), s, a);
+}
+
 }  // namespace
 
 int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_t* id_a, uint32_t* key_b,
               int32_t* id_b, const SortScratch& sc, int32_t* status, cudaStream_t s) {
     if (n <= 0) return MSC_OK;
+    if (n <= kOrderCoopMax) {
+        const CoopOrderArgs a{f, (uint32_t)n, order, {key_a, key_b},
+                              {reinterpret_cast<uint32_t*>(id_a), reinterpret_cast<uint32_t*>(id_b)}, sc.ord_cnt, status};
+        return ceil_div(n, CoopSmem<uint32_t, 8>::kTile) <= 2 * current_device().sms ? launch_coop<8>(a, s) : launch_coop<16>(a, s);
+    }
     Range rg;
     rg.n = n;
     rg.tiles = ceil_div(n, kTile);
@@ -516,9 +623,9 @@ int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_
     const int sms = current_device().sms;
     int occ = 0;
     {
-        int rr = configure_down<false, false, 8>();
+        int rr = configure_down<false, kOutSorted, 8>();
         if (rr) return rr;
-        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ord_down<false, false, 8>, kT, kDownSmem));
+        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ord_down<false, kOutSorted, 8>, kT, kDownSmem));
     }
     const int down_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * std::max(occ, 1));
     const int up_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * 4);
@@ -539,7 +646,7 @@ int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_
     a.vals_out = id_a;
     a.total = totals;
     a.use_tma = aligned16(f);
-    if ((r = launch_down<true, false, 0>(a, down_blocks, s, "order.down_first"))) return r;
+    if ((r = launch_down<true, kOutSorted, 0>(a, down_blocks, s, "order.down_first"))) return r;
     // pass 1: a -> b
     if ((r = launch_up<false, 8>(nullptr, key_a, rg, up_blocks, cnt, totals + kB, status, s))) return r;
     a.keys_in = key_a;
@@ -548,7 +655,7 @@ int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_
     a.vals_out = id_b;
     a.total = totals + kB;
     a.use_tma = aligned16(key_a) && aligned16(id_a);
-    if ((r = launch_down<false, false, 8>(a, down_blocks, s, "order.down"))) return r;
+    if ((r = launch_down<false, kOutSorted, 8>(a, down_blocks, s, "order.down"))) return r;
     // pass 2: b -> a
     if ((r = launch_up<false, 16>(nullptr, key_b, rg, up_blocks, cnt, totals + 2 * kB, status, s))) return r;
     a.keys_in = key_b;
@@ -557,19 +664,23 @@ int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_
     a.vals_out = id_a;
     a.total = totals + 2 * kB;
     a.use_tma = aligned16(key_b) && aligned16(id_b);
-    if ((r = launch_down<false, false, 16>(a, down_blocks, s, "order.down"))) return r;
+    if ((r = launch_down<false, kOutSorted, 16>(a, down_blocks, s, "order.down"))) return r;
     // pass 3: a -> (id, position) pairs filed by id bucket into (id_b, key_b)
     if ((r = launch_up<false, 24>(nullptr, key_a, rg, up_blocks, cnt, totals + 3 * kB, status, s))) return r;
     a.keys_in = key_a;
     a.vals_in = id_a;
     a.keys_out = nullptr;
+    a.total = totals + 3 * kB;
+    a.use_tma = aligned16(key_a) && aligned16(id_a);
+    if (n <= kOrderDirectMax) {
+        a.vals_out = order;
+        return launch_down<false, kOutOrder, 24>(a, down_blocks, s, "order.down_direct");
+    }
     a.vals_out = id_b;
     a.pair_pos = key_b;
     a.bucket_fill = fill;
     a.bucket_shift = order_bucket_shift(n);
-    a.total = totals + 3 * kB;
-    a.use_tma = aligned16(key_a) && aligned16(id_a);
-    if ((r = launch_down<false, true, 24>(a, down_blocks, s, "order.down_last"))) return r;
+    if ((r = launch_down<false, kOutBuckets, 24>(a, down_blocks, s, "order.down_last"))) return r;
     // the inverse permutation; the last pass's inputs are free
     return order_invert(a.bucket_shift, id_b, key_b, id_a, key_a, sc.sub_fill, n, order, status, s);
 }
