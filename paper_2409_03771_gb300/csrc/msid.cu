@@ -32,6 +32,7 @@
 
 #include <algorithm>
 
+#include "coop.cuh"
 #include "msid.cuh"
 #include "radix.cuh"
 
@@ -529,80 +530,113 @@ __global__ void __launch_bounds__(kRankThreads, 2) k_ms_chunk_rank(const unsigne
     }
 }
 
-// Route (b): compact occupied slots into (key, slot) pairs: each thread
-// scans 8 consecutive slots with 16-byte loads; one atomic append per
-// block chunk.
+// Route (b) in one cooperative launch: compact the occupied slots into
+// (key, slot) pairs (each thread scans 8 consecutive slots with 16-byte
+// loads, one atomic append per block and chunk), radix-sort the pairs by key
+// and write table_vals[slot] = rank of the slot's key.  As separate launches
+// the five to seven passes over the few thousand to few million pairs of a
+// usual field took some 20 us each, nearly all of it launch and look-back
+// latency (64^3 field with noise: 93 us as nine launches, 45 as one).  Only as many blocks as there are tiles of
+// pairs take part in the sort; a single tile needs no barrier at all.
 constexpr int kCompactPer = 8;
+constexpr int kPairItems = 8;
+using PairSmem = CoopSmem<unsigned long long, kPairItems>;
 
-__global__ void __launch_bounds__(kThreads) k_ms_compact(const unsigned long long* __restrict__ keys,
-                                                         uint32_t* ctl, unsigned long long* ukeys,
-                                                         int32_t* uvals, int32_t* status) {
-    __shared__ uint32_t s_warp[kThreads / 32];
+struct PairArgs {
+    const unsigned long long* table;
+    uint32_t* ctl;
+    unsigned long long* keys[2];
+    int32_t* slots[2];
+    uint32_t* vals;
+    int npass;
+    int keep_keys;      // the caller reads the sorted keys
+    uint32_t* scratch;  // kCoopScratchWords, then two barrier words
+    int32_t* status;
+};
+
+__global__ void __launch_bounds__(kCoopThreads) k_ms_pairs(const PairArgs a) {
+    extern __shared__ __align__(16) uint8_t pair_smem[];
+    PairSmem& S = *reinterpret_cast<PairSmem*>(pair_smem);
+    __shared__ uint32_t s_warp[kCoopWarps];
     __shared__ uint32_t s_base;
-    if (ctl[kCtlRoute] == 0u) return;
-    const int64_t slots = (int64_t)ctl[2] + kPad;
+    if (a.ctl[kCtlRoute] == 0u) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int64_t kChunkSlots = (int64_t)kThreads * kCompactPer;
-    const int64_t nchunks = (slots + kChunkSlots - 1) / kChunkSlots;
-    for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-        const int64_t i0 = c * kChunkSlots + (int64_t)tid * kCompactPer;
-        unsigned long long k[kCompactPer];
-        if (i0 + kCompactPer <= slots) {  // cap and kPad are multiples of 8: whole groups
+    {
+        const int64_t slots = (int64_t)a.ctl[2] + kPad;
+        constexpr int64_t kChunkSlots = (int64_t)kCoopThreads * kCompactPer;
+        const int64_t nchunks = (slots + kChunkSlots - 1) / kChunkSlots;
+        for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
+            const int64_t i0 = c * kChunkSlots + (int64_t)tid * kCompactPer;
+            unsigned long long k[kCompactPer];
+            if (i0 + kCompactPer <= slots) {  // cap and kPad are multiples of 8: whole groups
 #pragma unroll
-            for (int q = 0; q < kCompactPer / 2; ++q) {
-                const ulonglong2 v = reinterpret_cast<const ulonglong2*>(keys + i0)[q];
-                k[2 * q] = v.x;
-                k[2 * q + 1] = v.y;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < kCompactPer; ++j) k[j] = i0 + j < slots ? keys[i0 + j] : kEmpty;
-        }
-        uint32_t cnt = 0;
-#pragma unroll
-        for (int j = 0; j < kCompactPer; ++j) cnt += k[j] != kEmpty;
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t run = 0;
-            for (int w = 0; w < kThreads / 32; ++w) {
-                const uint32_t t = s_warp[w];
-                s_warp[w] = run;
-                run += t;
-            }
-            s_base = run ? atomicAdd(&ctl[kCtlCompact], run) : 0u;
-        }
-        __syncthreads();
-        uint32_t pos = s_base + s_warp[warp] + incl - cnt;
-#pragma unroll
-        for (int j = 0; j < kCompactPer; ++j) {
-            if (k[j] != kEmpty) {
-                MSC_GUARD(pos < (uint32_t)slots, status, -131) {
-                    ukeys[pos] = k[j];
-                    uvals[pos] = (int32_t)(i0 + j);
+                for (int q = 0; q < kCompactPer / 2; ++q) {
+                    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(a.table + i0)[q];
+                    k[2 * q] = v.x;
+                    k[2 * q + 1] = v.y;
                 }
-                ++pos;
+            } else {
+#pragma unroll
+                for (int j = 0; j < kCompactPer; ++j) k[j] = i0 + j < slots ? a.table[i0 + j] : kEmpty;
             }
+            uint32_t cnt = 0;
+#pragma unroll
+            for (int j = 0; j < kCompactPer; ++j) cnt += k[j] != kEmpty;
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane == 31) s_warp[warp] = incl;
+            __syncthreads();
+            if (tid == 0) {
+                uint32_t run = 0;
+                for (int w = 0; w < kCoopWarps; ++w) {
+                    const uint32_t t = s_warp[w];
+                    s_warp[w] = run;
+                    run += t;
+                }
+                s_base = run ? atomicAdd(&a.ctl[kCtlCompact], run) : 0u;
+            }
+            __syncthreads();
+            uint32_t pos = s_base + s_warp[warp] + incl - cnt;
+#pragma unroll
+            for (int j = 0; j < kCompactPer; ++j) {
+                if (k[j] != kEmpty) {
+                    MSC_GUARD(pos < (uint32_t)slots, a.status, -131) {
+                        a.keys[0][pos] = k[j];
+                        a.slots[0][pos] = (int32_t)(i0 + j);
+                    }
+                    ++pos;
+                }
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
-}
-
-// Route (b): table_vals[slot] = rank of the slot's key.
-__global__ void k_ms_rank(const int32_t* __restrict__ slots, const uint32_t* ctl, uint32_t* vals,
-                          int32_t* status) {
-    if (ctl[kCtlRoute] == 0u) return;
-    const int64_t K = ctl[kCtlCompact];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K;
-         i += (int64_t)gridDim.x * blockDim.x)
-        MSC_GUARD((uint32_t)slots[i] < ctl[2] + kPad, status, -132)
-        vals[slots[i]] = (uint32_t)i;
+    GridBarrier all{a.scratch + kCoopScratchWords, gridDim.x, 0};
+    if (!grid_barrier(all, a.status)) return;
+    const uint32_t K = __ldcg(a.ctl + kCtlCompact);
+    const uint32_t active = min(gridDim.x, (K + PairSmem::kTile - 1) / PairSmem::kTile);
+    if (blockIdx.x >= active) return;
+    GridBarrier bar{a.scratch + kCoopScratchWords + 1, active, 0};
+#pragma unroll 1
+    for (int p = 0; p < a.npass; ++p) {
+        const bool last = p + 1 == a.npass;
+        const unsigned long long* kin = a.keys[p & 1];
+        const int32_t* vin = a.slots[p & 1];
+        unsigned long long* kout = a.keys[(p & 1) ^ 1];
+        int32_t* vout = a.slots[(p & 1) ^ 1];
+        const CoopPass r = coop_radix_pass<unsigned long long, kPairItems>(
+            S, K, 8 * p, false, [&](uint32_t i) { return kin[i]; }, [&](uint32_t i) { return (uint32_t)vin[i]; },
+            [&](uint32_t pos, unsigned long long k, uint32_t slot) {
+                if (!last || a.keep_keys) kout[pos] = k;
+                if (!last) vout[pos] = (int32_t)slot;
+                else a.vals[slot] = pos;
+            },
+            a.scratch, bar, a.status);
+        if (r == kPassFailed) return;
+    }
 }
 
 // ms[v] = vals[ms[v]]: 8 vertices per thread, lane-consecutive, so the
@@ -710,51 +744,67 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
         k_ms_insert<<<grid_for(ceil_div(n, kInsJ)), kThreads, 0, s>>>(asc, desc, n, sc.table_keys, sc.ctl, ms, status);
     }
     MSC_LAUNCHED();
-    // route (a); each kernel returns at once on route (b).  The chunks cover
+    // route (a), unless the table always fits the cache; each kernel returns
+    // at once on route (b).  The chunks cover
     // the largest table; those past the one in use are empty.
-    const int64_t nchunks = chunks_for(sc.cap_max);
-    uint32_t* occ = sc.chunk;
-    uint32_t* occ_before = sc.chunk + nchunks;
-    {
-        TraceScope ts_("msid.occ", s);
-        k_ms_occ<<<grid_for(nchunks * kThreads, 8), kThreads, 0, s>>>(sc.table_keys, occ, nchunks, sc.ctl);
+    if (sc.cap_max > (int64_t)kCacheResidentSlots && !sorted_keys) {
+        const int64_t nchunks = chunks_for(sc.cap_max);
+        uint32_t* occ = sc.chunk;
+        uint32_t* occ_before = sc.chunk + nchunks;
+        {
+            TraceScope ts_("msid.occ", s);
+            k_ms_occ<<<grid_for(nchunks * kThreads, 8), kThreads, 0, s>>>(sc.table_keys, occ, nchunks, sc.ctl);
+        }
+        MSC_LAUNCHED();
+        {
+            TraceScope ts_("msid.chunk_scan", s);
+            k_ms_chunk_scan<<<1, kScanThreads, 0, s>>>(occ, occ_before, nchunks, sc.ctl);
+        }
+        MSC_LAUNCHED();
+        {
+            static int configured_dev = -1;
+            if (configured_dev != current_device().id) {
+                MSC_TRY(cudaFuncSetAttribute(k_ms_chunk_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRankSmem));
+                configured_dev = current_device().id;
+            }
+            TraceScope ts_("msid.chunk_rank", s);
+            const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nchunks, (int64_t)current_device().sms * 2));
+            k_ms_chunk_rank<<<grid, kRankThreads, kRankSmem, s>>>(sc.table_keys, sc.table_vals, occ_before, nchunks,
+                                                                   sc.ctl);
+        }
+        MSC_LAUNCHED();
     }
-    MSC_LAUNCHED();
+    // route (b), run when the flag asks for it (returns at once otherwise)
     {
-        TraceScope ts_("msid.chunk_scan", s);
-        k_ms_chunk_scan<<<1, kScanThreads, 0, s>>>(occ, occ_before, nchunks, sc.ctl);
-    }
-    MSC_LAUNCHED();
-    {
+        PairArgs a{};
+        a.table = sc.table_keys;
+        a.ctl = sc.ctl;
+        for (int i = 0; i < 2; ++i) {
+            a.keys[i] = sc.ukeys[i];
+            a.slots[i] = sc.uvals[i];
+        }
+        a.vals = sc.table_vals;
+        a.npass = std::max(1, (2 * sh + 7) / 8);
+        a.keep_keys = sorted_keys ? 1 : 0;
+        a.scratch = sc.sort.ord_cnt;
+        a.status = status;
         static int configured_dev = -1;
         if (configured_dev != current_device().id) {
-            MSC_TRY(cudaFuncSetAttribute(k_ms_chunk_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRankSmem));
+            MSC_TRY(cudaFuncSetAttribute(k_ms_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PairSmem)));
             configured_dev = current_device().id;
         }
-        TraceScope ts_("msid.chunk_rank", s);
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nchunks, (int64_t)current_device().sms * 2));
-        k_ms_chunk_rank<<<grid, kRankThreads, kRankSmem, s>>>(sc.table_keys, sc.table_vals, occ_before, nchunks,
-                                                               sc.ctl);
+        int blocks = 0;
+        const int r = coop_blocks(k_ms_pairs, kCoopThreads, sizeof(PairSmem),
+                                  std::min<int64_t>(ceil_div(n, PairSmem::kTile), kCoopMaxBlocks), &blocks);
+        if (r) return r;
+        MSC_TRY(cudaMemsetAsync(a.scratch + kCoopScratchWords, 0, 2 * sizeof(uint32_t), s));
+        {
+            TraceScope ts_("msid.pairs", s);
+            const int rr = coop_launch(k_ms_pairs, blocks, kCoopThreads, sizeof(PairSmem), s, a);
+            if (rr) return rr;
+        }
+        if (sorted_keys) *sorted_keys = sc.ukeys[a.npass & 1];
     }
-    MSC_LAUNCHED();
-    // route (b), run when the flag asks for it (every kernel returns at once otherwise)
-    {
-        TraceScope ts_("msid.compact", s);
-        k_ms_compact<<<grid_for((sc.cap_max + kPad) / kCompactPer, 4), kThreads, 0, s>>>(
-            sc.table_keys, sc.ctl, sc.ukeys[0], sc.uvals[0], status);
-    }
-    MSC_LAUNCHED();
-    bool in_alt = false;
-    int r = run_sort_u64(sc.ukeys[0], sc.uvals[0], sc.ukeys[1], sc.uvals[1],
-                         reinterpret_cast<const int32_t*>(sc.ctl + kCtlCompact), n + kPad, 2 * sh, sc.sort, status,
-                         s, &in_alt);
-    if (r) return r;
-    if (sorted_keys) *sorted_keys = in_alt ? sc.ukeys[1] : sc.ukeys[0];
-    {
-        TraceScope ts_("msid.rank", s);
-        k_ms_rank<<<grid_for(n), kThreads, 0, s>>>(in_alt ? sc.uvals[1] : sc.uvals[0], sc.ctl, sc.table_vals, status);
-    }
-    MSC_LAUNCHED();
     {
         TraceScope ts_("msid.lookup", s);
         k_ms_lookup<<<grid_for(n / kLookupPer + 1), kThreads, 0, s>>>(ms, n, sc.table_vals, sc.ctl, num_cells);

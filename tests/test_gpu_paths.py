@@ -141,3 +141,85 @@ def test_cc_mesh_row_orders(m, oracle_mod, n, edges, rows):
     row[1:] = np.cumsum(np.bincount(src, minlength=n))
     col = dst[at].astype(np.int32)
     np.testing.assert_array_equal(host(m.cc_mesh(cuda(row), cuda(col))), oracle_mod.cc_csr(row, col))
+
+
+# ---------------------------------------------------------------------------
+# vertex order: one cooperative launch, per-pass launches with a direct last
+# pass, per-pass launches with the inverse permutation
+
+
+def order_of(f):
+    perm = np.argsort(f + np.float32(0.0), kind="stable")
+    want = np.empty(f.size, np.int32)
+    want[perm] = np.arange(f.size, dtype=np.int32)
+    return want
+
+
+ORDER_SIZES = [2047, 2048, 2049, 64 * 2048, 64 * 2048 + 1, 304 * 2048, 304 * 2048 + 1, 304 * 4096 + 1, 1 << 21,
+               (1 << 21) + 1, 6144 * 700 + 5]
+
+
+@pytest.mark.parametrize("n", ORDER_SIZES)
+@pytest.mark.parametrize("kind", ["floats", "levels", "constant", "signs"])
+def test_order_sizes(m, n, kind):
+    rng = np.random.default_rng(n)
+    f = {"floats": lambda: rng.standard_normal(n), "levels": lambda: rng.integers(0, 256, n),
+         "constant": lambda: np.full(n, -2.5), "signs": lambda: rng.choice([-0.0, 0.0, -1.0, np.inf, -np.inf], n)}[kind]()
+    f = f.astype(np.float32)
+    np.testing.assert_array_equal(host(m.order(cuda(f))), order_of(f))
+
+
+@pytest.mark.parametrize("n", [(1 << 24), (1 << 24) + 1])
+def test_order_direct_limit(m, n):
+    f = np.random.default_rng(n).random(n, dtype=np.float32)
+    np.testing.assert_array_equal(host(m.order(cuda(f))), order_of(f))
+
+
+@pytest.mark.parametrize("n", [1, 2048, 5000, 700000, (1 << 21) + 7])
+def test_order_nan_anywhere(m, n):
+    for at in {0, n // 2, n - 1}:
+        f = torch.zeros(n, device="cuda")
+        f[at] = float("nan")
+        with pytest.raises(m.MSCError) as e:
+            m.order(f)
+        assert e.value.code == m.ERR_NAN
+
+
+# ---------------------------------------------------------------------------
+# pointer jumping: all sweeps in one launch, four or eight launches and a tail
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 1 << 20, (1 << 20) + 1, (1 << 24) - 1, 1 << 24])
+def test_compress_line(m, n):
+    """One path of n vertices: as many sweeps as any forest needs."""
+    p = (torch.arange(n, dtype=torch.int32, device="cuda") - 1).clamp_(min=0)
+    assert int(m.compress(p).max()) == 0
+
+
+@pytest.mark.parametrize("n", [3, 5000, (1 << 20) + 3, 1 << 24])
+def test_compress_long_cycle(m, n):
+    p = torch.arange(1, n + 1, dtype=torch.int32, device="cuda")
+    p[-1] = 0
+    with pytest.raises(m.MSCError) as e:
+        m.compress(p)
+    assert e.value.code == m.ERR_NOT_CONVERGED
+
+
+# ---------------------------------------------------------------------------
+# cell ids: pairs sorted by one block, by one tile per block, by several
+
+
+@pytest.mark.parametrize("n,roots", [(1, 1), (3000, 40), (20000, 45), (20000, 46), (70001, 300), (400000, 2000),
+                                     (3 << 20, 90000)])
+def test_ms_id_pair_counts(m, n, roots):
+    rng = np.random.default_rng(n + roots)
+    labels = []
+    for _ in range(2):
+        r = np.sort(rng.choice(n, roots, replace=False))
+        lab = r[rng.integers(0, roots, n)]
+        lab[r] = r
+        labels.append(lab.astype(np.int32))
+    keys, want = np.unique(labels[0].astype(np.int64) * n + labels[1], return_inverse=True)
+    ms, k = m.ms_id(*(cuda(x) for x in labels))
+    assert k == keys.size
+    np.testing.assert_array_equal(host(ms), want)
