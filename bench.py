@@ -233,18 +233,18 @@ def algorithmic_bytes(label, n, nm, nnz):
         "order.down_first": 12 * n,      # read f, write (key, id)
         "order.down": 16 * n,            # read and write (key, id)
         "order.down_last": 16 * n,       # read (key, id), write (id, position) pairs
-        "order.split": 16 * n,           # read the pairs, write them by sub-bucket of 2^15 ids
-        "order.scatter": 12 * n,         # read the pairs, write order
+        "order.down_direct": 12 * n,     # read (key, id), write order
+        "order.permute": 12 * n,         # read the pairs, write order
         "steepest.grid": 12 * n,         # read order, write asc + desc
         "msid.insert": 12 * n,           # read asc + desc, write slot
         "msid.lookup": 8 * n,            # read slot, write id
         "cc.local": 5 * n,               # read mask, write label
-        "cc.flatten": 8 * n,             # read label, write label
         "mesh.init": 4 * nm,             # write label = v
         "mesh.link": 24 * nm,            # read row[v], row[v+1], two columns, write two hooks
         "mesh.flatten": 8 * nm,          # read and write every label
-        # order.scan, the MS-id table passes (occupancy, chunk ranks) and
-        # mesh.hook move data-dependent amounts: no fixed algorithmic figure
+        # order.scan, the MS-id table passes (occupancy, chunk ranks),
+        # cc.flatten (labels of masked voxels only) and mesh.hook move
+        # data-dependent amounts: no fixed algorithmic figure
     }
     return table.get(label)
 

@@ -26,7 +26,7 @@
 //               completed in L2 before they are written back.
 // The last pass files (vertex id, position) pairs into buckets of
 // consecutive ids instead of writing sorted keys, and the order field is
-// their inverse permutation (k_pair_split / k_pair_scatter_local); while the
+// their inverse permutation (k_pair_permute); while the
 // order array fits the L2 it scatters the positions itself.  Small fields go
 // through all four passes in one cooperative launch (k_ord_coop).
 #include <cuda_runtime.h>
@@ -70,6 +70,35 @@ struct Range {
     int supers;
 };
 
+// The buffers of a sort and what its keys have in common.  varies[0] is the
+// OR of all keys and varies[1] the OR of their complements (written by the
+// first pass's upsweep): a byte that is the same in every key is zero in
+// their AND, and its pass moves nothing (the low mantissa bytes of small
+// whole numbers: an 8-bit scan takes two passes instead of four).  The
+// passes that do move alternate between the buffers, starting from the field.
+struct Buffers {
+    const float* f;
+    uint32_t* key[2];
+    int32_t* id[2];
+    const uint32_t* varies;
+    int aligned[3];  // 16-byte aligned: buffer 0, buffer 1, the field
+};
+
+__device__ __forceinline__ bool pass_moves(const Buffers& b, int p) {
+    return p == 3 || ((b.varies[0] & b.varies[1]) >> (8 * p) & 255u) != 0u;  // the last pass writes the result
+}
+
+__device__ __forceinline__ uint32_t* key_of(const Buffers& b, int i) { return i ? b.key[1] : b.key[0]; }
+__device__ __forceinline__ int32_t* id_of(const Buffers& b, int i) { return i ? b.id[1] : b.id[0]; }
+
+// Buffer holding the keys before pass p (-1: the field); the pass writes the
+// other one (0 after the field).
+__device__ __forceinline__ int source_of(const Buffers& b, int p) {
+    const uint32_t v = b.varies[0] & b.varies[1];
+    const int moved = (p > 0 && (v & 0xffu)) + (p > 1 && (v & 0xff00u)) + (p > 2 && (v & 0xff0000u));
+    return moved == 0 ? -1 : (moved - 1) & 1;
+}
+
 // The 8-bit digit of a key at a compile-time bit offset (one byte permute).
 template <int SHIFT>
 __device__ __forceinline__ uint32_t digit_of(uint32_t k) {
@@ -80,56 +109,82 @@ __device__ __forceinline__ uint32_t digit_of(uint32_t k) {
 
 // Upsweep: per-super-tile counts of the digit at SHIFT, stored digit-major
 // (cnt[d * kOrderMaxSuper + s]), plus the pass totals (one atomic per block
-// and digit).  FROM_F: the keys are made from the float field, whose NaNs
-// are reported here.
-template <bool FROM_F, int SHIFT>
-__global__ void __launch_bounds__(kT) k_ord_up(const float* __restrict__ f, const uint32_t* __restrict__ keys,
-                                               const Range r, uint32_t* __restrict__ cnt,
-                                               uint32_t* __restrict__ total, int32_t* status) {
+// and digit).  The first pass also reports NaNs and gathers `varies`.
+// Bound: the shared-memory atomics of the counts (LSU 69 %); 512^3: 0.12 ms
+// per pass, reading the keys alone takes 0.08.
+template <int SHIFT>
+__global__ void __launch_bounds__(kT, 4) k_ord_up(const Buffers bufs, const Range r, uint32_t* __restrict__ cnt,
+                                               uint32_t* __restrict__ total, uint32_t* varies, int32_t* status) {
     __shared__ uint32_t sh[kW * kB];
+    if (SHIFT > 0 && !pass_moves(bufs, SHIFT / 8)) return;
+    const int from = SHIFT == 0 ? -1 : source_of(bufs, SHIFT / 8);
+    const bool ff = from < 0;  // keys are made from the float field
+    uint32_t any1 = 0, all1 = ~0u, lo = ~0u, hi = 0;  // the first pass's keys
     const int tid = threadIdx.x, warp = tid >> 5;
     uint32_t* wh = sh + warp * kB;
-    bool nan = false;
     uint32_t mine = 0;  // this block's total of digit tid
-    const bool vec = FROM_F || ((uintptr_t)keys & 15) == 0;
-    constexpr int64_t kStep = (int64_t)kT * kHistRun;
+    const uint32_t* src = ff ? reinterpret_cast<const uint32_t*>(bufs.f) : key_of(bufs, from);
+    const bool vec = ((uintptr_t)src & 15) == 0;
     for (int s = blockIdx.x; s < r.supers; s += gridDim.x) {
         for (int i = tid; i < kW * kB; i += kT) sh[i] = 0;
         __syncthreads();
         const int64_t k0 = (int64_t)s * r.per_super * kTile;
         const int64_t k1 = min(r.n, k0 + r.per_super * kTile);
-        // two groups of 16 consecutive keys per thread and step: both groups'
-        // loads are in flight before either is counted
-        for (int64_t i0 = k0 + (int64_t)tid * kHistRun; i0 < k1; i0 += 2 * kStep) {
-            uint32_t a[kHistRun], b[kHistRun];
-            const int ca = (int)min((int64_t)kHistRun, k1 - i0);
-            const int cb = (int)max((int64_t)0, min((int64_t)kHistRun, k1 - i0 - kStep));
-            if constexpr (FROM_F) {
-                load_float_keys16(f, i0, ca, a, nan);
-                if (cb > 0) load_float_keys16(f, i0 + kStep, cb, b, nan);
-            } else {
+        // sixteen keys per thread and step in four lane-consecutive groups of
+        // four, the next step's loads in flight while one is counted
+        constexpr int kStep4 = kT * 16;
+        auto load = [&](int64_t base, uint32_t (&k)[16]) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t(&k)[kHistRun] = h ? b : a;
-                    const int c = h ? cb : ca;
-                    const int64_t j0 = i0 + h * kStep;
-                    if (c == kHistRun && vec) {
+            for (int q = 0; q < 4; ++q) {
+                const int64_t i = base + (int64_t)(q * kT + tid) * 4;
+                if (vec && i + 4 <= k1) {
+                    const uint4 v = __ldcs(reinterpret_cast<const uint4*>(src + i));
+                    k[4 * q] = v.x;
+                    k[4 * q + 1] = v.y;
+                    k[4 * q + 2] = v.z;
+                    k[4 * q + 3] = v.w;
+                } else {
 #pragma unroll
-                        for (int q = 0; q < kHistRun / 4; ++q) {
-                            const uint4 v = __ldcs(reinterpret_cast<const uint4*>(keys + j0) + q);
-                            k[4 * q] = v.x;
-                            k[4 * q + 1] = v.y;
-                            k[4 * q + 2] = v.z;
-                            k[4 * q + 3] = v.w;
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < kHistRun; ++j) k[j] = j < c ? keys[j0 + j] : 0u;
-                    }
+                    for (int j = 0; j < 4; ++j) k[4 * q + j] = i + j < k1 ? src[i + j] : 0u;
                 }
             }
-            count_runs_at(a, ca, SHIFT, wh);
-            if (cb > 0) count_runs_at(b, cb, SHIFT, wh);
+        };
+        uint32_t a[16];
+        if (k0 < k1) load(k0, a);
+        for (int64_t b = k0; b < k1; b += kStep4) {
+            uint32_t nx[16];
+            if (b + kStep4 < k1) load(b + kStep4, nx);
+            if (SHIFT == 0 || ff) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) a[j] = float_key(__uint_as_float(a[j]));
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t i = b + (int64_t)(q * kT + tid) * 4;
+                const int cnt = (int)max((int64_t)0, min((int64_t)4, k1 - i));
+                uint32_t cur = 0, run = 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j >= cnt) break;
+                    const uint32_t w = a[4 * q + j];
+                    if constexpr (SHIFT == 0) {
+                        any1 |= w;
+                        all1 &= w;
+                        lo = min(lo, w);
+                        hi = max(hi, w);
+                    }
+                    const uint32_t d = digit_of<SHIFT>(w);
+                    if (j > 0 && d != cur) {
+                        atomicAdd(&wh[cur], run);
+                        run = 0;
+                    }
+                    cur = d;
+                    ++run;
+                }
+                if (cnt > 0) atomicAdd(&wh[cur], run);
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) a[j] = nx[j];
         }
         __syncthreads();
         uint32_t c = 0;
@@ -139,15 +194,25 @@ __global__ void __launch_bounds__(kT) k_ord_up(const float* __restrict__ f, cons
         mine += c;
         __syncthreads();
     }
-    if (nan) record_error(status, MSC_ERR_NAN);
     if (mine) atomicAdd(&total[tid], mine);
+    if (SHIFT == 0) {
+        // a NaN's key lies above that of +Inf or below that of -Inf
+        if (hi > 0xff800000u || lo < 0x007fffffu) record_error(status, MSC_ERR_NAN);
+        any1 = __reduce_or_sync(0xffffffffu, any1);
+        all1 = __reduce_and_sync(0xffffffffu, all1);
+        if ((tid & 31) == 0) {
+            atomicOr(&varies[0], any1);
+            atomicOr(&varies[1], ~all1);
+        }
+    }
 }
 
 // Scan: block d takes digit d.  Its super-tiles' counts become exclusive
 // output positions starting at the digit's global start (the sum of the
 // totals of the smaller digits); warp w scans the w-th eighth of the row.
-__global__ void __launch_bounds__(kT) k_ord_scan(uint32_t* __restrict__ cnt, const uint32_t* __restrict__ total,
-                                                 int supers) {
+__global__ void __launch_bounds__(kT) k_ord_scan(const Buffers bufs, int pass, uint32_t* __restrict__ cnt,
+                                                 const uint32_t* __restrict__ total, int supers) {
+    if (!pass_moves(bufs, pass)) return;
     __shared__ uint32_t s_w[kW];
     __shared__ uint32_t s_g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -202,18 +267,13 @@ enum { kOutSorted, kOutBuckets, kOutOrder };
 constexpr int64_t kOrderDirectMax = 1 << 24;
 
 struct DownArgs {
-    const float* f;            // pass 0: the field (keys made from it, ids implicit)
-    const uint32_t* keys_in;   // other passes
-    const int32_t* vals_in;
-    uint32_t* keys_out;
-    int32_t* vals_out;         // BUCKET: the ids of the filed pairs
-    uint32_t* pair_pos;        // BUCKET: the positions of the filed pairs
-    uint32_t* bucket_fill;     // BUCKET: slots taken per id bucket (stride kOrderFillStride)
-    int bucket_shift;          // BUCKET: log2 of the ids per bucket
+    Buffers bufs;
+    int32_t* order;            // kOutOrder
+    uint32_t* bucket_fill;     // kOutBuckets: slots taken per id bucket (stride kOrderFillStride)
+    int bucket_shift;          // kOutBuckets: log2 of the ids per bucket
     Range r;
     const uint32_t* base;      // [256][kOrderMaxSuper] first output position per digit and super-tile
     const uint32_t* total;     // [256] keys per digit in this pass
-    int use_tma;               // the inputs are 16-byte aligned: full tiles come by bulk copy
     int32_t* status;
 };
 
@@ -221,13 +281,16 @@ struct DownArgs {
 // warp histograms (16-bit; after the count, each warp's tile-local start),
 // per-digit words, scan scratch, bucket words, two mbarriers.
 constexpr size_t kBufWords = 2 * kTile;
-constexpr size_t kDownSmem = 2 * kBufWords * 4 + kW * kB * 2 + 2 * kB * 4 + 32 * 4 + 2 * kB * 4 + 2 * 8;
+constexpr size_t kDownSmem = 2 * kBufWords * 4 + kW * kB * 2 + 2 * kB * 4 + 32 * 4 + 2 * kB * 4 + 2 * 8 + kW * kB * 4;
 
 // Lanes of the warp holding the same digit as this lane: one match
 // instruction, whose cost grows with the number of distinct digits in the
-// warp, or eight ballots, whose cost does not (digit_peers in radix.cuh).
+// warp, or a word of shared memory per digit (rank_in_warp), which a few
+// digits would crowd.  The middle passes of a 512^3 field took 1.62 ms with
+// eight ballots per key (issue-bound) and take 1.39 this way (LSU 79 %, DRAM
+// half busy); shares of the keys by ballots were no faster (1.41 to 1.5).
 
-template <bool FROM_F, int OUT, int SHIFT>
+template <int OUT, int SHIFT>
 __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     uint32_t* buf = reinterpret_cast<uint32_t*>(smem);                     // [2][kTile words | kTile words]
@@ -238,13 +301,18 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     uint32_t* s_bcnt = s_misc + 32;                                        // [kB] BUCKET
     uint32_t* s_bbase = s_bcnt + kB;                                       // [kB] BUCKET
     uint64_t* mbar = reinterpret_cast<uint64_t*>(s_bbase + kB);            // [2]
+    uint32_t* s_match = reinterpret_cast<uint32_t*>(mbar + 2);             // [kW][kB]
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Range r = a.r;
-    if ((int)blockIdx.x >= r.supers) return;  // block-uniform
+    if ((int)blockIdx.x >= r.supers || !pass_moves(a.bufs, SHIFT / 8)) return;  // block-uniform
+    const int from = SHIFT == 0 ? -1 : source_of(a.bufs, SHIFT / 8), to = from == 0;
+    const bool ff = from < 0;  // keys from the float field, ids implicit
+    constexpr bool FF = SHIFT == 0;
+    uint32_t* keys_out = key_of(a.bufs, to);  // kOutBuckets: the positions of the filed pairs
+    int32_t* vals_out = id_of(a.bufs, to);    // ... and their ids
     // few populated digits in this pass (a float field's top byte): rank
-    // with match, which is then cheaper than eight ballots (measured: 0.74
-    // against 0.92 ms for the top byte of a 512^3 field)
+    // with match
     const bool use_match = __syncthreads_count(a.total[tid] != 0u) <= MSC_ORD_MATCH_MAX;
     const int64_t G = gridDim.x;
     // the tiles of this block in processing order: super-tiles
@@ -255,6 +323,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
         return s < r.supers ? s * r.per_super : -1;
     };
     for (int i = tid; i < kW * kB / 2; i += kT) reinterpret_cast<uint32_t*>(s_wh)[i] = 0u;
+    for (int i = tid; i < kW * kB; i += kT) s_match[i] = 0u;
     if (tid == 0) {
         mbar_init(&mbar[0], 1);
         mbar_init(&mbar[1], 1);
@@ -262,15 +331,17 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     }
     __syncthreads();
 
-    const uint32_t* src_k = FROM_F ? reinterpret_cast<const uint32_t*>(a.f) : a.keys_in;
+    const uint32_t* src_k = ff ? reinterpret_cast<const uint32_t*>(a.bufs.f) : key_of(a.bufs, from);
+    const int32_t* src_v = ff ? nullptr : id_of(a.bufs, from);
+    const bool use_tma = ff ? a.bufs.aligned[2] : from ? a.bufs.aligned[1] : a.bufs.aligned[0];
     // full, aligned tiles come by bulk copy; the ragged last tile by plain loads
-    auto by_tma = [&](int64_t t) { return a.use_tma && (t + 1) * kTile <= r.n; };
+    auto by_tma = [&](int64_t t) { return use_tma && (t + 1) * kTile <= r.n; };
     auto issue = [&](int64_t t, int slot) {  // one thread
         if (t < 0 || !by_tma(t)) return;
         uint32_t* dst = buf + slot * kBufWords;
-        mbar_expect_tx(&mbar[slot], FROM_F ? kTile * 4 : kTile * 8);
+        mbar_expect_tx(&mbar[slot], ff ? kTile * 4 : kTile * 8);
         bulk_load(dst, src_k + t * kTile, kTile * 4, &mbar[slot]);
-        if constexpr (!FROM_F) bulk_load(dst + kTile, a.vals_in + t * kTile, kTile * 4, &mbar[slot]);
+        if (!ff) bulk_load(dst + kTile, src_v + t * kTile, kTile * 4, &mbar[slot]);
     };
     int64_t t = (int64_t)blockIdx.x * r.per_super;
     if (tid == 0) issue(t, 0);
@@ -304,13 +375,20 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
         } else {
             for (int i = tid; i < cnt; i += kT) {
                 bk[i] = src_k[tb + i];
-                if constexpr (!FROM_F) bv[i] = (uint32_t)a.vals_in[tb + i];
+                if (!ff) bv[i] = (uint32_t)src_v[tb + i];
+            }
+            __syncthreads();
+        }
+        if (!FF && ff) {  // the field after passes that moved nothing: make the pairs in place
+            for (int i = tid; i < cnt; i += kT) {
+                bk[i] = float_key(__uint_as_float(bk[i]));
+                bv[i] = (uint32_t)(tb + i);
             }
             __syncthreads();
         }
         auto key_at = [&](int li) -> uint32_t {
             const uint32_t w = bk[li];
-            return FROM_F ? float_key(__uint_as_float(w)) : w;
+            return FF ? float_key(__uint_as_float(w)) : w;
         };
         // stable rank among the warp's equal digits: earlier keys of the warp
         // (its 16-bit counter) + lower lanes of this step
@@ -326,16 +404,17 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
                 const bool valid = FULL || li < cnt;
                 const uint32_t d = valid ? digit_of<SHIFT>(key_at(li)) : 0u;
                 dg[k / 4] = (k & 3) ? (dg[k / 4] | d << (8 * (k & 3))) : d;
-                uint32_t peers;
-                if constexpr (MATCH) peers = __match_any_sync(0xffffffffu, valid ? d : 0x100u | lane);
-                else if constexpr (FULL) peers = digit_peers_all(d);
-                else peers = digit_peers(d, valid);
-                const uint32_t lower = __popc(peers & lt);
-                const uint32_t before = wh[d];
-                if (valid && lower == 0) wh[d] = (uint16_t)(before + __popc(peers));
-                const uint32_t rank = before + lower;
+                uint32_t rank;
+                if constexpr (MATCH) {
+                    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 0x100u | lane);
+                    const uint32_t lower = __popc(peers & lt), before = wh[d];
+                    if (valid && lower == 0) wh[d] = (uint16_t)(before + __popc(peers));
+                    rank = before + lower;
+                    __syncwarp();
+                } else {
+                    rank = rank_in_warp(d, valid, 1u << lane, lt, s_match + warp * kB, wh);
+                }
                 rk[k / 2] = (k & 1) ? (rk[k / 2] | rank << 16) : rank;
-                __syncwarp();
             }
         };
         if (cnt == kTile) {
@@ -367,7 +446,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
             // values into registers first (the field pass makes them from the
             // index), so that bv is free for the staged keys
             uint32_t val[kI];
-            if constexpr (!FROM_F) {
+            if constexpr (!FF) {
 #pragma unroll
                 for (int k = 0; k < kI; ++k) val[k] = bv[wb + 32 * k];
                 __syncthreads();
@@ -393,7 +472,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
                 const int li = wb + 32 * k;
                 if (li < cnt) {
                     const uint32_t lpos = (rk[k / 2] >> (16 * (k & 1))) & 0xffffu;
-                    MSC_GUARD(lpos < (uint32_t)kTile, a.status, -141) bk[lpos] = FROM_F ? (uint32_t)(tb + li) : val[k];
+                    MSC_GUARD(lpos < (uint32_t)kTile, a.status, -141) bk[lpos] = FF ? (uint32_t)(tb + li) : val[k];
                 }
             }
             __syncthreads();
@@ -405,8 +484,8 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
                     const uint32_t kk = bv[i];
                     const uint32_t pos = s_delta[digit_of<SHIFT>(kk)] + (uint32_t)i;
                     MSC_GUARD(pos < (uint64_t)r.n, a.status, -142) {
-                        a.keys_out[pos] = kk;
-                        a.vals_out[pos] = (int32_t)bk[i];
+                        keys_out[pos] = kk;
+                        vals_out[pos] = (int32_t)bk[i];
                     }
                 }
             }
@@ -418,7 +497,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
                     const uint32_t d = (dg[k / 4] >> (8 * (k & 3))) & 255u;
                     const uint32_t pos = s_delta[d] + wh[d] + ((rk[k / 2] >> (16 * (k & 1))) & 0xffffu);
                     const uint32_t id = bv[li];
-                    MSC_GUARD(id < (uint64_t)r.n && pos < (uint64_t)r.n, a.status, -146) a.vals_out[id] = (int32_t)pos;
+                    MSC_GUARD(id < (uint64_t)r.n && pos < (uint64_t)r.n, a.status, -146) a.order[id] = (int32_t)pos;
                 }
             }
             __syncwarp();
@@ -474,8 +553,8 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
                 const uint32_t slot_ = s_bbase[b] + ((uint32_t)i - s_bcnt[b]);
                 const uint32_t pos = bk[i];
                 MSC_GUARD(slot_ < (uint64_t)r.n && pos < (uint64_t)r.n, a.status, -145) {
-                    a.vals_out[slot_] = (int32_t)v;
-                    a.pair_pos[slot_] = pos;
+                    vals_out[slot_] = (int32_t)v;
+                    keys_out[slot_] = pos;
                 }
             }
         }
@@ -486,43 +565,56 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     }
 }
 
-template <bool FROM_F, int OUT, int SHIFT>
+template <int OUT, int SHIFT>
 int configure_down() {
     static int configured_dev = -1;  // the attribute is set once per device
     if (configured_dev != current_device().id) {
-        MSC_TRY(cudaFuncSetAttribute(k_ord_down<FROM_F, OUT, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kDownSmem));
+        MSC_TRY(cudaFuncSetAttribute(k_ord_down<OUT, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDownSmem));
         configured_dev = current_device().id;
     }
     return MSC_OK;
 }
 
-template <bool FROM_F, int OUT, int SHIFT>
-int launch_down(const DownArgs& a, int blocks, cudaStream_t s, const char* label) {
-    const int rc = configure_down<FROM_F, OUT, SHIFT>();
+// One digit pass: upsweep, scan, downsweep.
+struct PassLaunch {
+    DownArgs a;
+    uint32_t* cnt;
+    uint32_t* totals;  // [4][256]
+    uint32_t* varies;
+    int up_blocks, down_blocks;
+    cudaStream_t s;
+};
+
+template <int OUT, int SHIFT>
+int launch_pass(PassLaunch& p, const char* label) {
+    const int rc = configure_down<OUT, SHIFT>();
     if (rc) return rc;
+    uint32_t* total = p.totals + SHIFT / 8 * kB;
     {
-        TraceScope ts_(label, s);
-        k_ord_down<FROM_F, OUT, SHIFT><<<blocks, kT, kDownSmem, s>>>(a);
+        TraceScope ts_("order.up", p.s);
+        k_ord_up<SHIFT><<<p.up_blocks, kT, 0, p.s>>>(p.a.bufs, p.a.r, p.cnt, total, p.varies, p.a.status);
+    }
+    MSC_LAUNCHED();
+    {
+        TraceScope ts_("order.scan", p.s);
+        k_ord_scan<<<kB, kT, 0, p.s>>>(p.a.bufs, SHIFT / 8, p.cnt, total, p.a.r.supers);
+    }
+    MSC_LAUNCHED();
+    p.a.total = total;
+    {
+        TraceScope ts_(label, p.s);
+        k_ord_down<OUT, SHIFT><<<p.down_blocks, kT, kDownSmem, p.s>>>(p.a);
     }
     MSC_LAUNCHED();
     return MSC_OK;
 }
 
-template <bool FROM_F, int SHIFT>
-int launch_up(const float* f, const uint32_t* keys, const Range& rg, int blocks, uint32_t* cnt, uint32_t* total,
-              int32_t* status, cudaStream_t s) {
-    {
-        TraceScope ts_("order.up", s);
-        k_ord_up<FROM_F, SHIFT><<<blocks, kT, 0, s>>>(f, keys, rg, cnt, total, status);
-    }
-    MSC_LAUNCHED();
-    {
-        TraceScope ts_("order.scan", s);
-        k_ord_scan<<<kB, kT, 0, s>>>(cnt, total, rg.supers);
-    }
-    MSC_LAUNCHED();
-    return MSC_OK;
+// order[id] = position for the pairs the last pass has filed: into the
+// buffer after the one it read.
+__global__ void __launch_bounds__(kPermuteThreads) k_ord_permute(const Buffers bufs, int64_t n, int32_t* __restrict__ order,
+                                                                 int32_t* status) {
+    const int b = source_of(bufs, 3) == 0;
+    permute_pairs(id_of(bufs, b), key_of(bufs, b), n, b ? bufs.aligned[1] : bufs.aligned[0], order, status);
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
@@ -586,7 +678,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_ord_coop(const CoopOrderArgs a
 // thread while that leaves one tile per block at two blocks per SM (262 144:
 // 48 us, 61 with sixteen; 10^6: 93 and 76).
 constexpr int64_t kOrderCoopMax = 1 << 21;
-static_assert(kCoopScratchWords + 1 <= kOrderCntWords, "the barrier word follows the counts");
+static_assert(kCoopScratchWords + 2 <= kOrderCntWords, "the barrier words follow the counts");
 
 template <int ITEMS>
 int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
@@ -623,66 +715,40 @@ int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_
     const int sms = current_device().sms;
     int occ = 0;
     {
-        int rr = configure_down<false, kOutSorted, 8>();
+        int rr = configure_down<kOutSorted, 8>();
         if (rr) return rr;
-        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ord_down<false, kOutSorted, 8>, kT, kDownSmem));
+        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ord_down<kOutSorted, 8>, kT, kDownSmem));
     }
-    const int down_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * std::max(occ, 1));
-    const int up_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * 4);
-    uint32_t* cnt = sc.ord_cnt;
-    uint32_t* totals = sc.ord_cnt + (size_t)kB * kOrderMaxSuper;  // [4][256]
-    uint32_t* fill = totals + 4 * kB;
-    MSC_TRY(cudaMemsetAsync(totals, 0, (4 * kB + kOrderMaxBuckets * kOrderFillStride) * sizeof(uint32_t), s));
-
-    DownArgs a{};
+    PassLaunch p{};
+    p.down_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * std::max(occ, 1));
+    p.up_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * 4);
+    p.s = s;
+    p.cnt = sc.ord_cnt;
+    p.totals = sc.ord_cnt + (size_t)kB * kOrderMaxSuper;
+    uint32_t* fill = p.totals + 4 * kB;
+    p.varies = fill + kOrderMaxBuckets * kOrderFillStride;
+    MSC_TRY(cudaMemsetAsync(p.totals, 0, (4 * kB + kOrderMaxBuckets * kOrderFillStride + 2) * sizeof(uint32_t), s));
+    DownArgs& a = p.a;
+    a.bufs = Buffers{f, {key_a, key_b}, {id_a, id_b}, p.varies,
+                     {aligned16(key_a) && aligned16(id_a), aligned16(key_b) && aligned16(id_b), aligned16(f)}};
     a.r = rg;
-    a.base = cnt;
+    a.base = p.cnt;
     a.status = status;
-    a.f = f;
-    int r;
-    // pass 0: f -> (key_a, id_a)
-    if ((r = launch_up<true, 0>(f, nullptr, rg, up_blocks, cnt, totals, status, s))) return r;
-    a.keys_out = key_a;
-    a.vals_out = id_a;
-    a.total = totals;
-    a.use_tma = aligned16(f);
-    if ((r = launch_down<true, kOutSorted, 0>(a, down_blocks, s, "order.down_first"))) return r;
-    // pass 1: a -> b
-    if ((r = launch_up<false, 8>(nullptr, key_a, rg, up_blocks, cnt, totals + kB, status, s))) return r;
-    a.keys_in = key_a;
-    a.vals_in = id_a;
-    a.keys_out = key_b;
-    a.vals_out = id_b;
-    a.total = totals + kB;
-    a.use_tma = aligned16(key_a) && aligned16(id_a);
-    if ((r = launch_down<false, kOutSorted, 8>(a, down_blocks, s, "order.down"))) return r;
-    // pass 2: b -> a
-    if ((r = launch_up<false, 16>(nullptr, key_b, rg, up_blocks, cnt, totals + 2 * kB, status, s))) return r;
-    a.keys_in = key_b;
-    a.vals_in = id_b;
-    a.keys_out = key_a;
-    a.vals_out = id_a;
-    a.total = totals + 2 * kB;
-    a.use_tma = aligned16(key_b) && aligned16(id_b);
-    if ((r = launch_down<false, kOutSorted, 16>(a, down_blocks, s, "order.down"))) return r;
-    // pass 3: a -> (id, position) pairs filed by id bucket into (id_b, key_b)
-    if ((r = launch_up<false, 24>(nullptr, key_a, rg, up_blocks, cnt, totals + 3 * kB, status, s))) return r;
-    a.keys_in = key_a;
-    a.vals_in = id_a;
-    a.keys_out = nullptr;
-    a.total = totals + 3 * kB;
-    a.use_tma = aligned16(key_a) && aligned16(id_a);
-    if (n <= kOrderDirectMax) {
-        a.vals_out = order;
-        return launch_down<false, kOutOrder, 24>(a, down_blocks, s, "order.down_direct");
-    }
-    a.vals_out = id_b;
-    a.pair_pos = key_b;
+    a.order = order;
     a.bucket_fill = fill;
     a.bucket_shift = order_bucket_shift(n);
-    if ((r = launch_down<false, kOutBuckets, 24>(a, down_blocks, s, "order.down_last"))) return r;
-    // the inverse permutation; the last pass's inputs are free
-    return order_invert(a.bucket_shift, id_b, key_b, id_a, key_a, sc.sub_fill, n, order, status, s);
+    int r;
+    if ((r = launch_pass<kOutSorted, 0>(p, "order.down_first"))) return r;
+    if ((r = launch_pass<kOutSorted, 8>(p, "order.down"))) return r;
+    if ((r = launch_pass<kOutSorted, 16>(p, "order.down"))) return r;
+    if (n <= kOrderDirectMax) return launch_pass<kOutOrder, 24>(p, "order.down_direct");
+    if ((r = launch_pass<kOutBuckets, 24>(p, "order.down_last"))) return r;
+    {
+        TraceScope ts_("order.permute", s);
+        k_ord_permute<<<(unsigned)ceil_div(n, kPermuteChunk), kPermuteThreads, 0, s>>>(a.bufs, n, order, status);
+    }
+    MSC_LAUNCHED();
+    return MSC_OK;
 }
 
 }  // namespace msc

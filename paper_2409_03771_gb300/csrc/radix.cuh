@@ -141,4 +141,45 @@ __device__ __forceinline__ void count_runs_at(const KeyT (&k)[kHistRun], int cnt
     atomicAdd(&h[cur], run);
 }
 
+// Order inversion: order[id] = position for the (id, position) pairs filed by
+// id bucket.  The blocks in flight work on a few
+// neighbouring buckets, so the scattered stores fall into a window of some
+// megabytes that the L2 completes before it writes it back.  Bound: one L1
+// line per store (134M stores, 0.67 ms; their DRAM traffic takes 0.24).
+// Splitting the buckets further (2^15 ids) and scattering in shared memory
+// took 0.76 ms in two kernels.
+constexpr int kPermuteThreads = 256;
+constexpr int kPermutePer = 4;  // groups of four pairs per thread
+constexpr int kPermuteChunk = 4 * kPermutePer * kPermuteThreads;
+
+__device__ __forceinline__ void permute_pairs(const int32_t* __restrict__ ids, const uint32_t* __restrict__ pos, int64_t n,
+                                              bool vec, int32_t* __restrict__ order, int32_t* status) {
+    const int64_t c0 = (int64_t)blockIdx.x * kPermuteChunk + 4 * threadIdx.x;
+    int4 id[kPermutePer], p[kPermutePer];
+#pragma unroll
+    for (int q = 0; q < kPermutePer; ++q) {
+        const int64_t i = c0 + q * (4 * kPermuteThreads);
+        if (vec && i + 4 <= n) {
+            id[q] = __ldcs(reinterpret_cast<const int4*>(ids + i));
+            p[q] = __ldcs(reinterpret_cast<const int4*>(pos + i));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kPermutePer; ++q) {
+        const int64_t i = c0 + q * (4 * kPermuteThreads);
+        if (vec && i + 4 <= n) {
+            MSC_GUARD(max(max((uint32_t)id[q].x, (uint32_t)id[q].y), max((uint32_t)id[q].z, (uint32_t)id[q].w)) < (uint64_t)n,
+                      status, -108) {
+                order[id[q].x] = p[q].x;
+                order[id[q].y] = p[q].y;
+                order[id[q].z] = p[q].z;
+                order[id[q].w] = p[q].w;
+            }
+        } else {
+            for (int64_t j = i; j < min(n, i + 4); ++j)
+                MSC_GUARD((uint32_t)ids[j] < (uint64_t)n, status, -108) order[ids[j]] = (int32_t)pos[j];
+        }
+    }
+}
+
 }  // namespace msc

@@ -17,9 +17,7 @@
 // look-back array, sums its predecessors' counts and scatters through
 // shared memory.  The last pass of an order files (vertex id, position)
 // pairs into buckets of consecutive ids; the order field is their inverse
-// permutation, written through shared memory: the buckets are split into
-// sub-buckets of 2^15 ids, each scattered into one CTA's shared memory and
-// written out as whole lines (k_pair_split, k_pair_scatter_local).
+// permutation (k_pair_permute).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -416,201 +414,22 @@ __global__ void __launch_bounds__(kThreads, 3) k_onesweep(const PassArgs<KeyT> a
 }
 
 // Width of the id buckets the last pass files pairs into: 2^19 ids at
-// least (so that each bucket splits into 16 sub-buckets of 2^15), and at
-// most kMaxBuckets buckets.
+// least (2 MiB of the order array), and at most kMaxBuckets buckets.
 int bucket_shift(int64_t n) {
     return std::max(19, ceil_log2(ceil_div(std::max<int64_t>(n, 1), kMaxBuckets)));
 }
 
-// Two-level order inversion.  (1) k_pair_split: every
-// chunk of 4096 filed pairs (a chunk lies inside one bucket of 2^shift ids)
-// re-files its pairs into sub-buckets of 2^15 ids; sub-bucket j holds
-// exactly the ids j * 2^15 + [0, 2^15) and so fills those pair slots.  A
-// chunk reserves its share of each sub-bucket with one atomic per
-// sub-bucket and regroups its pairs in shared memory, so that each run is
-// written with consecutive lanes.  (2) k_pair_scatter_local: one CTA per
-// sub-bucket stores its 2^15 positions into a 128 KiB shared-memory slice
-// of the order array and writes the slice out as whole lines.
-constexpr int kSubLog2 = 15;
-constexpr int kSubIds = 1 << kSubLog2;
-constexpr int kSplitThreads = 512;
-constexpr int kSplitChunk = 4096;
-constexpr int kSplitPer = kSplitChunk / kSplitThreads;  // 8
-constexpr int kMaxSub = 1 << 8;  // sub-buckets per bucket (shift <= 23)
-
-// The chunk's pairs arrive by 1D TMA bulk copy into one half of a shared
-// double buffer while the previous chunk is filed (plain loads for a ragged
-// last chunk or unaligned arrays); they are counted per sub-bucket,
-// regrouped in place and written out as runs.
-constexpr size_t kSplitSmem = (size_t)2 * 2 * kSplitChunk * 4 + (2 * kMaxSub + 32) * 4 + 2 * 8;
-
-__global__ void __launch_bounds__(kSplitThreads, 2) k_pair_split(const int32_t* __restrict__ ids_in,
-                                                                 const uint32_t* __restrict__ pos_in, int64_t n,
-                                                                 int shift, int use_tma, uint32_t* sub_fill,
-                                                                 int32_t* __restrict__ ids_out,
-                                                                 uint32_t* __restrict__ pos_out, int32_t* status) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    uint32_t* buf = reinterpret_cast<uint32_t*>(smem);     // [2][ids kSplitChunk | positions kSplitChunk]
-    uint32_t* s_cnt = buf + 2 * 2 * kSplitChunk;            // [kMaxSub] counts, then chunk-local starts
-    uint32_t* s_base = s_cnt + kMaxSub;                     // [kMaxSub] first slot of the run in each sub-bucket
-    uint32_t* s_w = s_base + kMaxSub;                       // [32]
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(s_w + 32); // [2]
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nsub = 1 << (shift - kSubLog2);
-    const int64_t nchunks = (n + kSplitChunk - 1) / kSplitChunk;
-    if ((int64_t)blockIdx.x >= nchunks) return;  // block-uniform
-    if (tid == 0) {
-        mbar_init(&mbar[0], 1);
-        mbar_init(&mbar[1], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    auto by_tma = [&](int64_t c) { return use_tma && (c + 1) * kSplitChunk <= n; };
-    auto issue = [&](int64_t c, int slot) {  // one thread
-        if (c >= nchunks || !by_tma(c)) return;
-        uint32_t* dst = buf + slot * 2 * kSplitChunk;
-        mbar_expect_tx(&mbar[slot], 2 * kSplitChunk * 4);
-        bulk_load(dst, ids_in + c * kSplitChunk, kSplitChunk * 4, &mbar[slot]);
-        bulk_load(dst + kSplitChunk, pos_in + c * kSplitChunk, kSplitChunk * 4, &mbar[slot]);
-    };
-    if (tid == 0) issue(blockIdx.x, 0);
-    int it = 0;
-    for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x, ++it) {
-        const int slot = it & 1;
-        uint32_t* bi = buf + slot * 2 * kSplitChunk;
-        uint32_t* bp = bi + kSplitChunk;
-        if (tid == 0) issue(c + gridDim.x, slot ^ 1);
-        const int64_t c0 = c * kSplitChunk;
-        const int cnt = (int)min((int64_t)kSplitChunk, n - c0);
-        const int64_t s0 = (c0 >> shift) << shift;  // first id of the chunk's bucket
-        for (int i = tid; i < nsub; i += kSplitThreads) s_cnt[i] = 0;
-        if (by_tma(c)) {
-            const bool ok = mbar_wait(&mbar[slot], (uint32_t)(it >> 1) & 1u, kSpinLimit);
-            if (__syncthreads_or(!ok)) {  // a copy never landed: report, let the prefetch finish, stop
-                if (tid == 0) {
-                    record_error(status, MSC_ERR_INTERNAL);
-                    if (c + gridDim.x < nchunks && by_tma(c + gridDim.x))
-                        mbar_wait(&mbar[slot ^ 1], (uint32_t)((it + 1) >> 1) & 1u, kSpinLimit);
-                }
-                return;
-            }
-        } else {
-            for (int i = tid; i < cnt; i += kSplitThreads) {
-                bi[i] = (uint32_t)ids_in[c0 + i];
-                bp[i] = pos_in[c0 + i];
-            }
-            __syncthreads();
-        }
-        int32_t id[kSplitPer];
-        uint32_t ps[kSplitPer], rank[kSplitPer];
-#pragma unroll
-        for (int k = 0; k < kSplitPer; ++k) {
-            const int i = tid + k * kSplitThreads;
-            id[k] = -1;
-            if (i < cnt) {
-                id[k] = (int32_t)bi[i];
-                ps[k] = bp[i];
-                const int64_t off = (int64_t)id[k] - s0;
-                MSC_GUARD(off >= 0 && off < (int64_t(1) << shift), status, -106)
-                rank[k] = atomicAdd(&s_cnt[off >> kSubLog2], 1u);
-            }
-        }
-        __syncthreads();
-        // chunk-local exclusive starts over the nsub (<= 256) sub-buckets, and
-        // the chunk's reservation in each of them
-        const uint32_t cc = tid < nsub ? s_cnt[tid] : 0u;
-        uint32_t incl = cc;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) s_w[warp] = incl;
-        __syncthreads();
-        uint32_t before = 0;
-        for (int w = 0; w < warp; ++w) before += s_w[w];
-        if (tid < nsub) {
-            s_base[tid] = cc ? atomicAdd(&sub_fill[(s0 >> kSubLog2) + tid], cc) : 0u;
-            s_cnt[tid] = before + incl - cc;
-        }
-        __syncthreads();
-        // regroup in place: every pair of the chunk was read before the barriers above
-#pragma unroll
-        for (int k = 0; k < kSplitPer; ++k)
-            if (id[k] >= 0) {
-                const uint32_t j = s_cnt[(uint32_t)(id[k] - s0) >> kSubLog2] + rank[k];
-                MSC_GUARD(j < (uint32_t)kSplitChunk, status, -109) {
-                    bi[j] = (uint32_t)id[k];
-                    bp[j] = ps[k];
-                }
-            }
-        __syncthreads();
-        for (int i = tid; i < cnt; i += kSplitThreads) {
-            const int32_t v = (int32_t)bi[i];
-            const int sub = (int)((uint32_t)(v - s0) >> kSubLog2);
-            const uint32_t slot_ = s_base[sub] + (uint32_t)i - s_cnt[sub];
-            const int64_t dst = s0 + ((int64_t)sub << kSubLog2) + slot_;
-            MSC_GUARD(slot_ < (uint32_t)kSubIds && dst < n, status, -107) {
-                ids_out[dst] = v;
-                pos_out[dst] = bp[i];
-            }
-        }
-        // this buffer is refilled by a bulk copy (async proxy) two chunks on
-        fence_proxy_async_smem();
-        __syncthreads();
-    }
+__global__ void __launch_bounds__(kPermuteThreads) k_pair_permute(const int32_t* __restrict__ ids,
+                                                                  const uint32_t* __restrict__ pos, int64_t n, int vec,
+                                                                  int32_t* __restrict__ order, int32_t* status) {
+    permute_pairs(ids, pos, n, vec, order, status);
 }
 
-__global__ void __launch_bounds__(1024) k_pair_scatter_local(const int32_t* __restrict__ ids,
-                                                             const uint32_t* __restrict__ pos, int64_t n,
-                                                             int32_t* __restrict__ order, int32_t* status) {
-    extern __shared__ __align__(16) int32_t slice[];  // kSubIds
-    const int64_t nsub = (n + kSubIds - 1) >> kSubLog2;
-    for (int64_t sb = blockIdx.x; sb < nsub; sb += gridDim.x) {
-        const int64_t s0 = sb << kSubLog2, s1 = min(n, s0 + kSubIds);
-        const int cnt = (int)(s1 - s0);
-        for (int i = threadIdx.x; i < cnt; i += 1024) {
-            const int32_t id = __ldcs(ids + s0 + i);
-            const uint32_t p = __ldcs(pos + s0 + i);
-            const int64_t off = (int64_t)id - s0;
-            MSC_GUARD(off >= 0 && off < cnt, status, -108)
-            slice[off] = (int32_t)p;
-        }
-        __syncthreads();
-        // 16-byte stores when the caller's array allows them (s0 is a multiple
-        // of 2^15, so the base pointer decides), else one word at a time
-        const int full = ((uintptr_t)order & 15) == 0 ? cnt >> 2 : 0;
-        for (int i = threadIdx.x; i < full; i += 1024)
-            reinterpret_cast<int4*>(order + s0)[i] = reinterpret_cast<const int4*>(slice)[i];
-        for (int i = full * 4 + threadIdx.x; i < cnt; i += 1024) order[s0 + i] = slice[i];
-        __syncthreads();
-    }
-}
-
-int launch_pair_split_scatter(int shift, const int32_t* ids, const uint32_t* pos, int32_t* ids2, uint32_t* pos2,
-                              uint32_t* sub_fill, int64_t n, int32_t* order, int32_t* status, cudaStream_t s) {
-    const int sms = current_device().sms;
-    MSC_TRY(cudaMemsetAsync(sub_fill, 0, (size_t)(ceil_div(n, kSubIds) + 1) * sizeof(uint32_t), s));
-    static int configured_dev = -1;
-    if (configured_dev != current_device().id) {
-        MSC_TRY(cudaFuncSetAttribute(k_pair_scatter_local, cudaFuncAttributeMaxDynamicSharedMemorySize, kSubIds * 4));
-        MSC_TRY(cudaFuncSetAttribute(k_pair_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplitSmem));
-        configured_dev = current_device().id;
-    }
-    {
-        const int64_t chunks = ceil_div(n, kSplitChunk);
-        const int use_tma = ((uintptr_t)ids & 15) == 0 && ((uintptr_t)pos & 15) == 0;
-        TraceScope ts_("order.split", s);
-        k_pair_split<<<(unsigned)std::min<int64_t>(chunks, (int64_t)sms * 2), kSplitThreads, kSplitSmem, s>>>(
-            ids, pos, n, shift, use_tma, sub_fill, ids2, pos2, status);
-    }
-    MSC_LAUNCHED();
-    const int64_t nsub = ceil_div(n, kSubIds);
-    {
-        TraceScope ts_("order.scatter", s);
-        k_pair_scatter_local<<<(unsigned)std::min<int64_t>(nsub, (int64_t)sms), 1024, kSubIds * 4, s>>>(
-            ids2, pos2, n, order, status);
-    }
+int launch_pair_permute(const int32_t* ids, const uint32_t* pos, int64_t n, int32_t* order, int32_t* status,
+                        cudaStream_t s) {
+    const int vec = (((uintptr_t)ids | (uintptr_t)pos) & 15) == 0;
+    TraceScope ts_("order.permute", s);
+    k_pair_permute<<<(unsigned)ceil_div(n, kPermuteChunk), kPermuteThreads, 0, s>>>(ids, pos, n, vec, order, status);
     MSC_LAUNCHED();
     return MSC_OK;
 }
@@ -640,15 +459,9 @@ int launch_pass(const PassArgs<KeyT>& a, int64_t max_n, cudaStream_t s, const ch
 
 int order_bucket_shift(int64_t n) { return bucket_shift(n); }
 
-int order_invert(int shift, const int32_t* ids, const uint32_t* pos, int32_t* ids2, uint32_t* pos2,
-                 uint32_t* sub_fill, int64_t n, int32_t* order, int32_t* status, cudaStream_t s) {
-    return launch_pair_split_scatter(shift, ids, pos, ids2, pos2, sub_fill, n, order, status, s);
-}
-
 void size_sort_scratch(Sizer& s, int64_t n) {
     s.take<uint32_t>(kOrderCntWords);
     s.take<uint32_t>(8 * kBins + kCounterWords);
-    s.take<uint32_t>(ceil_div(std::max<int64_t>(n, 1), kSubIds) + 1);
     s.take<unsigned long long>((size_t)std::max<int64_t>(1, ceil_div(n, kSortTile)) * kBins);
 }
 
@@ -657,7 +470,6 @@ SortScratch carve_sort_scratch(Carver& c, int64_t n) {
     sc.ord_cnt = c.take<uint32_t>(kOrderCntWords);
     sc.hist = c.take<uint32_t>(8 * kBins + kCounterWords);
     sc.tile_counters = sc.hist + 8 * kBins;
-    sc.sub_fill = c.take<uint32_t>(ceil_div(std::max<int64_t>(n, 1), kSubIds) + 1);
     sc.max_tiles = std::max<int64_t>(1, ceil_div(n, kSortTile));
     sc.lookback = c.take<unsigned long long>((size_t)sc.max_tiles * kBins);
     return sc;
@@ -695,7 +507,6 @@ static int hist_grid(int64_t n) {
 
 void size_seg_sort_scratch(Sizer& s, int count, int64_t tiles) {
     s.take<uint32_t>((size_t)count * kSegPasses * kBins + kCounterWords);
-    s.take<uint32_t>(ceil_div(std::max<int64_t>(tiles, 1) * kSortTile, kSubIds) + 1);
     s.take<unsigned long long>((size_t)std::max<int64_t>(1, tiles) * kBins);
 }
 
@@ -705,7 +516,6 @@ SortScratch carve_seg_sort_scratch(Carver& c, int count, int64_t tiles) {
     const size_t hist_words = (size_t)count * kSegPasses * kBins;
     sc.hist = c.take<uint32_t>(hist_words + kCounterWords);
     sc.tile_counters = sc.hist + hist_words;
-    sc.sub_fill = c.take<uint32_t>(ceil_div(std::max<int64_t>(tiles, 1) * kSortTile, kSubIds) + 1);
     sc.max_tiles = std::max<int64_t>(1, tiles);
     sc.lookback = c.take<unsigned long long>((size_t)sc.max_tiles * kBins);
     return sc;
@@ -778,7 +588,7 @@ int run_order_seg(const float* f, const SegTable& t, int32_t* order, uint32_t* k
     a.tile_counter = sc.tile_counters + 3;
     a.epoch = 4;
     if ((r = launch_pass<uint32_t, false, true, true>(a, t.total, s, "order.pass_last"))) return r;
-    return launch_pair_split_scatter(a.bucket_shift, iout, kout, iin, kin, sc.sub_fill, t.total, order, status, s);
+    return launch_pair_permute(iout, kout, t.total, order, status, s);
 }
 
 int run_sort_u64(unsigned long long* keys, int32_t* vals, unsigned long long* keys_alt,

@@ -223,3 +223,25 @@ def test_ms_id_pair_counts(m, n, roots):
     ms, k = m.ms_id(*(cuda(x) for x in labels))
     assert k == keys.size
     np.testing.assert_array_equal(host(ms), want)
+
+
+@pytest.mark.parametrize("n", [5000, 300000, (1 << 21) + 4099, (1 << 24) + 12345])
+@pytest.mark.parametrize("bytes_", [(), (0,), (1,), (2,), (3,), (0, 2), (1, 3), (2, 3), (0, 1, 2)])
+def test_order_constant_bytes(m, n, bytes_):
+    """Keys that differ in some bytes only: the passes of the others move nothing."""
+    rng = np.random.default_rng(n + len(bytes_))
+    bits = np.full(n, 0x3f123456, np.uint32)
+    for b in bytes_:
+        r = rng.integers(0, 256 if b < 2 else 64, n, dtype=np.uint32) << np.uint32(8 * b)
+        bits = (bits & ~np.uint32(0xff << (8 * b))) | r
+    f = bits.view(np.float32)
+    np.testing.assert_array_equal(host(m.order(cuda(f))), order_of(f))
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_order_unaligned_field_large(m, shift):
+    n = (1 << 21) + 6144 * 3 + 5
+    f = np.random.default_rng(shift).integers(0, 200, n).astype(np.float32)  # the field is read by a later pass too
+    buf = torch.empty(n + shift, device="cuda")
+    buf[shift:] = cuda(f)
+    np.testing.assert_array_equal(host(m.order(buf[shift:])), order_of(f))
