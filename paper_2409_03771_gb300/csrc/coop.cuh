@@ -89,26 +89,6 @@ struct CoopSmem {
     uint32_t w[8];
 };
 
-// Stable rank of this lane's digit among the warp's earlier keys (counter
-// wh) and lower lanes: the lanes of each digit meet in a word of shared
-// memory (one atomic OR and one load instead of eight ballots).  Leaves
-// match cleared.
-__device__ __forceinline__ uint32_t rank_in_warp(uint32_t d, bool valid, uint32_t lane_bit, uint32_t lt, uint32_t* match,
-                                                 uint16_t* wh) {
-    if (valid) atomicOr(&match[d], lane_bit);
-    __syncwarp();
-    const uint32_t peers = valid ? match[d] : 0u;
-    const uint32_t before = wh[d];
-    __syncwarp();
-    const uint32_t lower = __popc(peers & lt);
-    if (valid && lower == 0) {
-        match[d] = 0;
-        wh[d] = (uint16_t)(before + __popc(peers));
-    }
-    __syncwarp();
-    return before + lower;
-}
-
 enum CoopPass { kPassFailed, kPassMoved, kPassSkipped };
 
 // One digit pass over n keys by the blocks 0 .. bar.blocks - 1.  key(i) and

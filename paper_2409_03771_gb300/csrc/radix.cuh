@@ -48,29 +48,25 @@ __device__ __forceinline__ uint32_t block_scan_256(uint32_t v, uint32_t* s_w) {
     return v;
 }
 
-// Lanes of the warp whose 8-bit digit equals this lane's (valid lanes
-// only), from eight ballots -- no match instruction, no divergence.
-__device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid) {
-    uint32_t eq = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-        eq &= bit ? bal : ~bal;
+// Stable rank of this lane's digit among the warp's earlier keys (counter
+// wh) and lower lanes: the lanes of each digit meet in a word of shared
+// memory (one atomic OR and one load instead of eight ballots).  Leaves
+// match cleared.
+template <typename CountT>
+__device__ __forceinline__ uint32_t rank_in_warp(uint32_t d, bool valid, uint32_t lane_bit, uint32_t lt, uint32_t* match,
+                                                 CountT* wh) {
+    if (valid) atomicOr(&match[d], lane_bit);
+    __syncwarp();
+    const uint32_t peers = valid ? match[d] : 0u;
+    const uint32_t before = wh[d];
+    __syncwarp();
+    const uint32_t lower = __popc(peers & lt);
+    if (valid && lower == 0) {
+        match[d] = 0;
+        wh[d] = (CountT)(before + __popc(peers));
     }
-    return eq;
-}
-
-// The same for a warp whose 32 lanes all hold a valid digit.
-__device__ __forceinline__ uint32_t digit_peers_all(uint32_t d) {
-    uint32_t eq = 0xffffffffu;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-        eq &= bit ? bal : ~bal;
-    }
-    return eq;
+    __syncwarp();
+    return before + lower;
 }
 
 constexpr int kHistRun = 16;  // consecutive keys per thread in the histogram

@@ -245,3 +245,18 @@ def test_order_unaligned_field_large(m, shift):
     buf = torch.empty(n + shift, device="cuda")
     buf[shift:] = cuda(f)
     np.testing.assert_array_equal(host(m.order(buf[shift:])), order_of(f))
+
+
+# ---------------------------------------------------------------------------
+# 64-bit key sorts (adjacency): histogram steps of 4096 keys, warps of one digit
+
+
+@pytest.mark.parametrize("dims", [(31, 5, 4), (64, 40, 33), (129, 65, 67)])
+@pytest.mark.parametrize("bound", [2, 255, 1 << 20])
+@pytest.mark.parametrize("conn", [6, 14])
+def test_adjacency_key_counts(m, oracle_mod, dims, bound, conn):
+    n = dims[0] * dims[1] * dims[2]
+    lab = np.random.default_rng(n + bound).integers(0, bound, n).astype(np.int32)
+    got = m.adjacency_grid(cuda(lab), dims, conn, label_bound=bound)
+    for g, w in zip(got, oracle_mod.adjacency_grid(lab, dims, conn)):
+        np.testing.assert_array_equal(host(g), w)
