@@ -148,7 +148,9 @@ __global__ void __launch_bounds__(kThreads) k_ms_vote(const int32_t* __restrict_
                                                       uint32_t* ctl) {
     if (ctl[2] <= kCacheResidentSlots) return;
     const int t = blockIdx.x * kThreads + threadIdx.x;
-    const uint32_t a = (uint32_t)asc[(int64_t)t * n / kHubSamples];
+    // hashed places: evenly spaced ones can all fall on one face of the grid,
+    // where neighbours share their minimum
+    const uint32_t a = (uint32_t)asc[(int64_t)(((mix64(t + 1) >> 32) * (unsigned long long)n) >> 32)];
     if (atomicAdd(&votes[(a * 0x9E3779B1u) >> 18], 1u) + 1 == kHubVotes) ctl[kCtlRoute] = ctl[kCtlHome] = 1u;
 }
 
