@@ -348,6 +348,19 @@ def _finish(status: torch.Tensor, where: str):
     _check(code, where)
 
 
+def _status_and_count(dev):
+    """Addresses of a status and a count word, and the tensor that holds
+    both: one read back (and one synchronisation) brings the two."""
+    both = torch.empty(2, dtype=torch.int32, device=dev)
+    return both.data_ptr(), both.data_ptr() + 4, both
+
+
+def _finish_count(both: torch.Tensor, where: str) -> int:
+    code, count = both.tolist()  # synchronises the stream
+    _check(code, where)
+    return count
+
+
 def _ws(op: int, n: int, dev, nnz: int = 0) -> torch.Tensor:
     return torch.empty(max(msc_workspace_bytes(op, n, nnz), 1), dtype=torch.uint8, device=dev)
 
@@ -419,12 +432,10 @@ def ms_id(asc: torch.Tensor, desc: torch.Tensor):
     d = _flat(desc, torch.int32)
     n = a.numel()
     ms = torch.empty(n, dtype=torch.int32, device=dev)
-    k = torch.empty(1, dtype=torch.int32, device=dev)
+    st, k, both = _status_and_count(dev)
     ws = _ws(OP_MS_ID, n, dev)
-    st = torch.empty(1, dtype=torch.int32, device=dev)
     _check(msc_ms_id(a, d, n, ms, k, ws, ws.numel(), st), "msc_ms_id")
-    _finish(st, "msc_ms_id")
-    return ms, int(k.item())
+    return ms, _finish_count(both, "msc_ms_id")
 
 
 def segment(f: torch.Tensor, dims, ws: torch.Tensor | None = None):
@@ -435,13 +446,11 @@ def segment(f: torch.Tensor, dims, ws: torch.Tensor | None = None):
     if n != int(dims[0]) * int(dims[1]) * int(dims[2]):
         raise MSCError(ERR_ARG, "segment: dims do not match the field size")
     outs = [torch.empty(n, dtype=torch.int32, device=dev) for _ in range(4)]
-    k = torch.empty(1, dtype=torch.int32, device=dev)
+    st, k, both = _status_and_count(dev)
     if ws is None:
         ws = _ws(OP_SEGMENT, n, dev)
-    st = torch.empty(1, dtype=torch.int32, device=dev)
     _check(msc_segment(f, dims, *outs, k, ws, ws.numel(), st), "msc_segment")
-    _finish(st, "msc_segment")
-    return (*outs, int(k.item()))
+    return (*outs, _finish_count(both, "msc_segment"))
 
 
 def cc_mask(mask: torch.Tensor, dims, conn: int = 6) -> torch.Tensor:

@@ -721,7 +721,7 @@ static int launch_emit(const EmitArgs& ea, int conn, int64_t tiles, cudaStream_t
     MSC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // persistent: as many CTAs as fit on the GPU at once
     int occ = 0;
-    MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem));
+    MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, smem));
     {
         TraceScope ts_("adjacency.emit", s);
         kern<<<blocks_for(tiles, std::max(occ, 1)), kThreads, smem, s>>>(ea);

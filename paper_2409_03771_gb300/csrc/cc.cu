@@ -740,7 +740,7 @@ int run_cc_mask(const uint8_t* mask, msc_grid gd, int conn, int32_t* label, int3
     auto local = mask8 ? k_cc_local<true> : k_cc_local<false>;
     auto merge = mask8 ? k_cc_merge<true> : k_cc_merge<false>;
     int occ = 1;
-    MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, local, kThreads, 0));
+    MSC_TRY(max_blocks_per_sm(&occ, local, kThreads, 0));
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)sms * std::max(occ, 1)));
     {
         TraceScope ts_("cc.local", s);

@@ -118,6 +118,16 @@ unsigned long long launch_count();
 // Properties of the current device (cached per device id).
 const Device& current_device();
 
+// Resident blocks per SM of a kernel on the current device.  The runtime
+// works this out anew on every call (1.5 us of host time, five to ten times
+// per segmentation), so the answers are remembered per device.
+cudaError_t max_blocks_per_sm(int* out, const void* kernel, int threads, size_t smem);
+
+template <typename K>
+cudaError_t max_blocks_per_sm(int* out, K* kernel, int threads, size_t smem) {
+    return max_blocks_per_sm(out, reinterpret_cast<const void*>(kernel), threads, smem);
+}
+
 // Bump-pointer carving of a caller workspace (256-byte aligned pieces).
 struct Carver {
     char* base;

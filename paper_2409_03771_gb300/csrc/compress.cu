@@ -309,7 +309,7 @@ CompressScratch carve_compress_scratch(Carver& c, int64_t n, int count) {
 int run_compress(int32_t* const* ptrs, int count, int32_t n, const CompressScratch& sc,
                  int32_t* status, cudaStream_t s, const CompressTune& tune) {
     if (n <= 0 || count < 1 || count > 2) return n < 0 ? MSC_ERR_ARG : MSC_OK;
-    MSC_TRY(cudaMemsetAsync(sc.ctl, 0, sizeof(JumpCtl) * count, s));
+    if (!tune.ctl_zeroed) MSC_TRY(cudaMemsetAsync(sc.ctl, 0, sizeof(JumpCtl) * count, s));
     JumpPair pr{};
     pr.n = n;
     pr.roots = tune.roots;
@@ -329,7 +329,7 @@ int run_compress(int32_t* const* ptrs, int count, int32_t n, const CompressScrat
     const int full = std::min(full_sweeps(n), steps);
     if (full > 0) {
         int occ = 1;
-        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0));
+        MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, 0));
         const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, (int64_t)current_device().sms * std::max(occ, 1)));
         for (int st = 0; st < full; ++st) {
             {

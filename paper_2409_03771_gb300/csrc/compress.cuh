@@ -21,6 +21,7 @@ struct CompressTune {
                              // most 1.5x its capacity (an overflow leaves a full sweep next)
     int build_shift = 3;     // fill_lists off: build it once <= n >> build_shift changed
     bool trusted = false;  // pointers from the stencil kernels: skip range / cycle tests
+    bool ctl_zeroed = false;    // the caller has cleared the scratch's ctl
     uint32_t* roots = nullptr;  // roots[i] += #self-pointers of array i (first sweep)
 };
 

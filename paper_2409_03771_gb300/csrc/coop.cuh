@@ -253,7 +253,7 @@ __device__ __forceinline__ CoopPass coop_radix_pass(CoopSmem<KeyT, ITEMS>& S, ui
 template <typename K>
 int coop_blocks(K kernel, int threads, size_t smem, int64_t want, int* out) {
     int occ = 0;
-    MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem));
+    MSC_TRY(max_blocks_per_sm(&occ, kernel, threads, smem));
     if (occ < 1) return MSC_ERR_CUDA;
     *out = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)current_device().sms * occ));
     return MSC_OK;

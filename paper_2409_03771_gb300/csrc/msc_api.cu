@@ -4,7 +4,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
+#include <tuple>
 
 #include "adjacency.cuh"
 #include "cc.cuh"
@@ -36,6 +38,26 @@ const Device& current_device() {
         }
     }
     return d;
+}
+
+cudaError_t max_blocks_per_sm(int* out, const void* kernel, int threads, size_t smem) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, int, size_t>, int> known;  // one entry per kernel and launch shape
+    const auto key = std::make_tuple(current_device().id, kernel, threads, smem);
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        const auto it = known.find(key);
+        if (it != known.end()) {
+            *out = it->second;
+            return cudaSuccess;
+        }
+    }
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, threads, smem);
+    if (e == cudaSuccess) {
+        std::lock_guard<std::mutex> lock(mu);
+        known[key] = *out;
+    }
+    return e;
 }
 
 bool make_tensor_map_3d(CUtensorMap* map, const void* base, int elem_bytes, int nx, int ny, int nz,
@@ -72,7 +94,13 @@ bool make_tensor_map_3d(CUtensorMap* map, const void* base, int elem_bytes, int 
 
 namespace {
 
-constexpr size_t kCommonWords = 64;  // uint32 control words shared by all stages
+// Control words of a segmentation, cleared by one fill: the cell ids' words
+// (the order's barrier among them), then the pointer jumping's.
+struct SegmentCtl {
+    uint32_t ms[kMsCtlWords];
+    JumpCtl jump[2];
+};
+constexpr int kOrderBarrier = 48;  // of the ms words: free until the cell ids
 
 // Workspaces are carved into 256-byte aligned pieces, some read with
 // 16-byte loads: the base must be 256-byte aligned.
@@ -96,7 +124,7 @@ void size_order(Sizer& s, int64_t n) {
 // Segment workspace: common words, then the largest of the three stages.
 size_t segment_bytes(int64_t n) {
     Sizer common;
-    common.take<uint32_t>(kCommonWords);
+    common.take<SegmentCtl>(1);
     Sizer sort, comp, ms;
     sort.take<int32_t>(std::max<int64_t>(n, 1));
     size_sort_scratch(sort, n);
@@ -217,9 +245,10 @@ int msc_segment(const float* f, msc_grid g, int32_t* order, int32_t* asc, int32_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     MSC_TRY(cudaMemsetAsync(d_status, 0, sizeof(int32_t), s));
     Carver c(ws, ws_bytes);
-    uint32_t* common = c.take<uint32_t>(kCommonWords);
+    SegmentCtl* ctl = c.take<SegmentCtl>(1);
+    uint32_t* common = ctl->ms;
     const size_t stage_off = c.used;
-    MSC_TRY(cudaMemsetAsync(common, 0, kCommonWords * sizeof(uint32_t), s));
+    MSC_TRY(cudaMemsetAsync(ctl, 0, sizeof(SegmentCtl), s));
     // 1. order; the asc / desc / ms outputs double as the sort's ping-pong
     {
         Carver st(ws, ws_bytes);
@@ -227,7 +256,7 @@ int msc_segment(const float* f, msc_grid g, int32_t* order, int32_t* asc, int32_
         int32_t* ib = st.take<int32_t>(n);
         SortScratch sc = carve_sort_scratch(st, n);
         int r = run_order(f, n, order, reinterpret_cast<uint32_t*>(asc), desc,
-                          reinterpret_cast<uint32_t*>(ms), ib, sc, d_status, s);
+                          reinterpret_cast<uint32_t*>(ms), ib, sc, d_status, s, common + kOrderBarrier);
         if (r) return r;
     }
     // 2. steepest pointers (the extrema are counted by the first jump sweep)
@@ -238,8 +267,10 @@ int msc_segment(const float* f, msc_grid g, int32_t* order, int32_t* asc, int32_
         Carver st(ws, ws_bytes);
         st.used = stage_off;
         CompressScratch sc = carve_compress_scratch(st, n, 2);
+        sc.ctl = ctl->jump;
         int32_t* arr[2] = {asc, desc};
         CompressTune tune;
+        tune.ctl_zeroed = true;
         tune.trusted = true;  // made by the stencil above: in range, acyclic
         tune.roots = common;  // common[0] = #minima (asc roots), common[1] = #maxima
         r = run_compress(arr, 2, (int32_t)n, sc, d_status, s, tune);

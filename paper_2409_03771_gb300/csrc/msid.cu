@@ -57,6 +57,7 @@ constexpr int kCtlM = 17;       // largest slot - asc * cap / n of a pair
 constexpr int kCtlCompact = 18; // route (b): compacted pairs
 constexpr int kCtlShift = 19;   // b of the pair keys
 constexpr int kCtlHome = 20;    // home slots of a table too big for the cache: 0 by the minimum, 1 by both labels
+constexpr int kCtlBarrier = 40; // two grid barriers of the pair sort, zero at its start
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
     // 64-bit finaliser of MurmurHash3
@@ -552,7 +553,7 @@ struct PairArgs {
     uint32_t* vals;
     int npass;
     int keep_keys;      // the caller reads the sorted keys
-    uint32_t* scratch;  // kCoopScratchWords, then two barrier words
+    uint32_t* scratch;  // kCoopScratchWords
     int32_t* status;
 };
 
@@ -616,12 +617,12 @@ __global__ void __launch_bounds__(kCoopThreads) k_ms_pairs(const PairArgs a) {
             __syncthreads();
         }
     }
-    GridBarrier all{a.scratch + kCoopScratchWords, gridDim.x, 0};
+    GridBarrier all{a.ctl + kCtlBarrier, gridDim.x, 0};
     if (!grid_barrier(all, a.status)) return;
     const uint32_t K = __ldcg(a.ctl + kCtlCompact);
     const uint32_t active = min(gridDim.x, (K + PairSmem::kTile - 1) / PairSmem::kTile);
     if (blockIdx.x >= active) return;
-    GridBarrier bar{a.scratch + kCoopScratchWords + 1, active, 0};
+    GridBarrier bar{a.ctl + kCtlBarrier + 1, active, 0};
 #pragma unroll 1
     for (int p = 0; p < a.npass; ++p) {
         const bool last = p + 1 == a.npass;
@@ -695,7 +696,7 @@ void size_ms_scratch(Sizer& s, int64_t n) {
         s.take<unsigned long long>(std::max<int64_t>(n, 1) + kPad);
         s.take<int32_t>(std::max<int64_t>(n, 1) + kPad);
     }
-    s.take<uint32_t>(64);
+    s.take<uint32_t>(kMsCtlWords);
     s.take<uint32_t>(2 * chunks_for(cap_max_for(n)));
     size_sort_scratch(s, n + kPad);
 }
@@ -709,7 +710,7 @@ MsScratch carve_ms_scratch(Carver& c, int64_t n) {
         sc.ukeys[i] = c.take<unsigned long long>(std::max<int64_t>(n, 1) + kPad);
         sc.uvals[i] = c.take<int32_t>(std::max<int64_t>(n, 1) + kPad);
     }
-    sc.ctl = c.take<uint32_t>(64);
+    sc.ctl = c.take<uint32_t>(kMsCtlWords);
     sc.chunk = c.take<uint32_t>(2 * chunks_for(sc.cap_max));
     sc.sort = carve_sort_scratch(c, n + kPad);
     return sc;
@@ -723,7 +724,7 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
         return MSC_OK;
     }
     const int sh = ms_pair_shift(n);
-    if (!counts_known) MSC_TRY(cudaMemsetAsync(sc.ctl, 0, 4 * sizeof(uint32_t), s));
+    if (!counts_known) MSC_TRY(cudaMemsetAsync(sc.ctl, 0, kMsCtlWords * sizeof(uint32_t), s));
     if (!counts_known) {
         TraceScope ts_("msid.prepare", s);
         k_ms_prepare<<<grid_for(n), kThreads, 0, s>>>(asc, desc, n, sc.ctl, status);
@@ -799,7 +800,6 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
         const int r = coop_blocks(k_ms_pairs, kCoopThreads, sizeof(PairSmem),
                                   std::min<int64_t>(ceil_div(n, PairSmem::kTile), kCoopMaxBlocks), &blocks);
         if (r) return r;
-        MSC_TRY(cudaMemsetAsync(a.scratch + kCoopScratchWords, 0, 2 * sizeof(uint32_t), s));
         {
             TraceScope ts_("msid.pairs", s);
             const int rr = coop_launch(k_ms_pairs, blocks, kCoopThreads, sizeof(PairSmem), s, a);

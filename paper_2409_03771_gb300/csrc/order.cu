@@ -631,7 +631,8 @@ struct CoopOrderArgs {
     int32_t* order;
     uint32_t* key[2];
     uint32_t* id[2];
-    uint32_t* scratch;  // kCoopScratchWords, then the barrier word
+    uint32_t* scratch;  // kCoopScratchWords
+    uint32_t* barrier;  // 0 at the start
     int32_t* status;
 };
 
@@ -639,7 +640,7 @@ template <int ITEMS>
 __global__ void __launch_bounds__(kCoopThreads) k_ord_coop(const CoopOrderArgs a) {
     extern __shared__ __align__(16) uint8_t coop_smem[];
     CoopSmem<uint32_t, ITEMS>& S = *reinterpret_cast<CoopSmem<uint32_t, ITEMS>*>(coop_smem);
-    GridBarrier bar{a.scratch + kCoopScratchWords, gridDim.x, 0};
+    GridBarrier bar{a.barrier, gridDim.x, 0};
     int src = -1;  // the buffer holding the keys; -1: the field
     bool nan = false;
 #pragma unroll 1
@@ -678,7 +679,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_ord_coop(const CoopOrderArgs a
 // thread while that leaves one tile per block at two blocks per SM (262 144:
 // 48 us, 61 with sixteen; 10^6: 93 and 76).
 constexpr int64_t kOrderCoopMax = 1 << 21;
-static_assert(kCoopScratchWords + 2 <= kOrderCntWords, "the barrier words follow the counts");
+static_assert(kCoopScratchWords + 1 <= kOrderCntWords, "the barrier word follows the counts");
 
 template <int ITEMS>
 int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
@@ -692,7 +693,6 @@ int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
     const int r = coop_blocks(k_ord_coop<ITEMS>, kCoopThreads, sizeof(Smem),
                               std::min<int64_t>(ceil_div(a.n, Smem::kTile), kCoopMaxBlocks), &blocks);
     if (r) return r;
-    MSC_TRY(cudaMemsetAsync(a.scratch + kCoopScratchWords, 0, sizeof(uint32_t), s));
     TraceScope ts_("order.coop", s);
     return coop_launch(k_ord_coop<ITEMS>, blocks, kCoopThreads, sizeof(Smem), s, a);
 }
@@ -700,11 +700,15 @@ int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
 }  // namespace
 
 int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_t* id_a, uint32_t* key_b,
-              int32_t* id_b, const SortScratch& sc, int32_t* status, cudaStream_t s) {
+              int32_t* id_b, const SortScratch& sc, int32_t* status, cudaStream_t s, uint32_t* barrier) {
     if (n <= 0) return MSC_OK;
     if (n <= kOrderCoopMax) {
+        if (!barrier) {
+            barrier = sc.ord_cnt + kCoopScratchWords;
+            MSC_TRY(cudaMemsetAsync(barrier, 0, sizeof(uint32_t), s));
+        }
         const CoopOrderArgs a{f, (uint32_t)n, order, {key_a, key_b},
-                              {reinterpret_cast<uint32_t*>(id_a), reinterpret_cast<uint32_t*>(id_b)}, sc.ord_cnt, status};
+                              {reinterpret_cast<uint32_t*>(id_a), reinterpret_cast<uint32_t*>(id_b)}, sc.ord_cnt, barrier, status};
         return ceil_div(n, CoopSmem<uint32_t, 8>::kTile) <= 2 * current_device().sms ? launch_coop<8>(a, s) : launch_coop<16>(a, s);
     }
     Range rg;
@@ -717,7 +721,7 @@ int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_
     {
         int rr = configure_down<kOutSorted, 8>();
         if (rr) return rr;
-        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ord_down<kOutSorted, 8>, kT, kDownSmem));
+        MSC_TRY(max_blocks_per_sm(&occ, k_ord_down<kOutSorted, 8>, kT, kDownSmem));
     }
     PassLaunch p{};
     p.down_blocks = (int)std::min<int64_t>(rg.supers, (int64_t)sms * std::max(occ, 1));

@@ -455,7 +455,7 @@ int launch_pass(const PassArgs<KeyT>& a, int64_t max_n, cudaStream_t s, const ch
         configured_dev = current_device().id;
     }
     int occ = 0;
-    MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem));
+    MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, smem));
     const int64_t ntiles = SEG ? a.seg_tiles : ceil_div(max_n, kSortTile);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)current_device().sms * std::max(occ, 1)));
     {

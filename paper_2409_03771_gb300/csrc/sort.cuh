@@ -32,9 +32,10 @@ SortScratch carve_sort_scratch(Carver& c, int64_t n);
 
 // order[v] = rank of (f[v], v).  Uses two (key, id) ping-pong buffers of n
 // entries each.  Records MSC_ERR_NAN in status when f holds a NaN.
+// `barrier` (optional): a word that is 0 now and free for this call.
 int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_t* id_a,
               uint32_t* key_b, int32_t* id_b, const SortScratch& sc, int32_t* status,
-              cudaStream_t s);
+              cudaStream_t s, uint32_t* barrier = nullptr);
 
 // Packed segments sorted independently (batched instances).  Segment i
 // holds keys [off[i], off[i+1]) and tiles [tile0[i], tile0[i+1]) of

@@ -479,7 +479,7 @@ int run_steepest_grid(const int32_t* order, msc_grid gd, int32_t* asc, int32_t* 
     if (tma) {
         auto kern = extrema ? (packed ? k_steepest_tma<int32_t, true> : k_steepest_tma<int64_t, true>)
                             : (packed ? k_steepest_tma<int32_t, false> : k_steepest_tma<int64_t, false>);
-        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0));
+        MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, 0));
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)sms * std::max(occ, 1)));
         {
             TraceScope ts_("steepest.grid", s);
@@ -488,7 +488,7 @@ int run_steepest_grid(const int32_t* order, msc_grid gd, int32_t* asc, int32_t* 
     } else {
         auto kern = extrema ? (packed ? k_steepest_ld<int32_t, true> : k_steepest_ld<int64_t, true>)
                             : (packed ? k_steepest_ld<int32_t, false> : k_steepest_ld<int64_t, false>);
-        MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0));
+        MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, 0));
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)sms * std::max(occ, 1)));
         {
             TraceScope ts_("steepest.grid", s);
@@ -511,7 +511,7 @@ int launch_batch(const int32_t* order, const BatchInst* inst, const int32_t* til
                  int64_t ntiles, bool packed, int32_t* asc, int32_t* desc, uint32_t* ext, cudaStream_t s) {
     auto kern = packed ? k_steepest_batch<int32_t, S> : k_steepest_batch<int64_t, S>;
     int occ = 1;
-    MSC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, 0));
+    MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, 0));
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)current_device().sms * std::max(occ, 1)));
     {
         TraceScope ts_("steepest.batch", s);
