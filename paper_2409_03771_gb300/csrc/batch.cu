@@ -14,7 +14,8 @@
 //      before those of instance i+1, so instance i's dense ids are the
 //      global ranks minus the number of pairs of earlier instances, found
 //      by a binary search of off_i * total in the sorted pair keys;
-//   5. a rebase pass turns packed ids into instance-local ones.
+//   5. a rebase pass looks the cell ids up and turns packed ids into
+//      instance-local ones.
 //
 // A plan captures steps 1-5 once as a CUDA graph; the autotuner times the
 // tile shape of step 2 and the active-list threshold of step 3.
@@ -233,26 +234,45 @@ __global__ void k_batch_first(const unsigned long long* __restrict__ keys, const
     num_cells[i] = (int32_t)(b - a);
 }
 
-// Packed ids -> instance-local ids, per sort tile (inside one instance).
-constexpr int kRebasePer = kSortTile / kThreads;  // 16
+// Packed ids -> instance-local ids, per sort tile (inside one instance); the
+// cell ids come from the table slots that the insert left in ms.  Four
+// vertices per thread and step, their loads in flight together.  Bound: DRAM
+// (24 bytes per vertex).  96 grids, 45M vertices: 378 us as a lookup and a
+// rebase with one vertex per step, 224 in one.
+constexpr int kRebasePer = 4;
 
 __global__ void __launch_bounds__(kThreads) k_batch_rebase(const int32_t* __restrict__ tile_seg,
                                                            const int32_t* __restrict__ off,
                                                            const int32_t* __restrict__ tile0,
-                                                           const int32_t* __restrict__ first, int64_t tiles,
-                                                           int32_t* ms, int32_t* asc, int32_t* desc) {
+                                                           const int32_t* __restrict__ first,
+                                                           const uint32_t* __restrict__ rank_of_slot, int64_t tiles,
+                                                           int32_t* __restrict__ ms, int32_t* __restrict__ asc,
+                                                           int32_t* __restrict__ desc) {
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int i = tile_seg[t];
         const int32_t o = off[i], n = off[i + 1] - o, fr = first[i];
-        const int64_t l0 = (t - tile0[i]) * kSortTile + threadIdx.x;
+        const int32_t l0 = (int32_t)(t - tile0[i]) * kSortTile + threadIdx.x;
+#pragma unroll 1
+        for (int s = 0; s < kSortTile; s += kRebasePer * kThreads) {
+            int32_t m[kRebasePer], a[kRebasePer], d[kRebasePer];
 #pragma unroll
-        for (int j = 0; j < kRebasePer; ++j) {
-            const int64_t l = l0 + j * kThreads;
-            if (l < n) {
-                const int64_t v = o + l;
-                ms[v] -= fr;
-                asc[v] -= o;
-                desc[v] -= o;
+            for (int j = 0; j < kRebasePer; ++j) {
+                const int32_t l = l0 + s + j * kThreads;
+                m[j] = l < n ? ms[o + l] : 0;
+                a[j] = l < n ? asc[o + l] : 0;
+                d[j] = l < n ? desc[o + l] : 0;
+            }
+#pragma unroll
+            for (int j = 0; j < kRebasePer; ++j)
+                if (l0 + s + j * kThreads < n) m[j] = (int32_t)rank_of_slot[m[j]];
+#pragma unroll
+            for (int j = 0; j < kRebasePer; ++j) {
+                const int32_t l = l0 + s + j * kThreads;
+                if (l < n) {
+                    ms[o + l] = m[j] - fr;
+                    asc[o + l] = a[j] - o;
+                    desc[o + l] = d[j] - o;
+                }
             }
         }
     }
@@ -327,28 +347,28 @@ int run_batch(void* ws, size_t ws_bytes, const Layout& L, const DevLayout& d, co
         if (r) return r;
     }
     // 4. packed cell ids, then per-instance first ranks and cell counts
-    const unsigned long long* keys = nullptr;
+    MsRanked ranked{};
     {
         Carver st(ws, ws_bytes);
         st.used = d.stage_off;
         MsScratch sc = carve_ms_scratch(st, L.total);
         sc.ctl = d.ctl;
         r = run_ms_id(B.asc, B.desc, total, B.ms, reinterpret_cast<int32_t*>(d.ctl + 4), sc, true, B.status, s,
-                      &keys);
+                      &ranked);
         if (r) return r;
     }
     {
         TraceScope ts_("batch.first", s);
         k_batch_first<<<(unsigned)ceil_div(L.count, kThreads), kThreads, 0, s>>>(
-            keys, d.ctl, d.off, L.count, ms_pair_shift(L.total), d.first, B.num_cells);
+            ranked.keys, d.ctl, d.off, L.count, ms_pair_shift(L.total), d.first, B.num_cells);
     }
     MSC_LAUNCHED();
     // 5. instance-local ids
     {
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(L.tiles, (int64_t)current_device().sms * 8));
         TraceScope ts_("batch.rebase", s);
-        k_batch_rebase<<<grid, kThreads, 0, s>>>(d.tile_seg, d.off, d.tile0, d.first, L.tiles, B.ms, B.asc,
-                                                 B.desc);
+        k_batch_rebase<<<grid, kThreads, 0, s>>>(d.tile_seg, d.off, d.tile0, d.first, ranked.rank_of_slot, L.tiles,
+                                                 B.ms, B.asc, B.desc);
     }
     MSC_LAUNCHED();
     return MSC_OK;

@@ -718,7 +718,7 @@ MsScratch carve_ms_scratch(Carver& c, int64_t n) {
 
 int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, int32_t* num_cells,
               const MsScratch& sc, bool counts_known, int32_t* status, cudaStream_t s,
-              const unsigned long long** sorted_keys) {
+              MsRanked* ranked) {
     if (n <= 0) {
         MSC_TRY(cudaMemsetAsync(num_cells, 0, sizeof(int32_t), s));
         return MSC_OK;
@@ -734,10 +734,10 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
         TraceScope ts_("msid.clear", s);
         // at least kHubCounters threads, so that every vote counter is cleared
         const int grid = std::max(grid_for(sc.cap_max + kPad, 4), kHubCounters / kThreads);
-        k_ms_clear<<<grid, kThreads, 0, s>>>(sc.table_keys, sc.table_vals, sc.ctl, n, sc.cap_max, sh, sorted_keys ? 1 : 0);
+        k_ms_clear<<<grid, kThreads, 0, s>>>(sc.table_keys, sc.table_vals, sc.ctl, n, sc.cap_max, sh, ranked ? 1 : 0);
     }
     MSC_LAUNCHED();
-    if (sc.cap_max > (int64_t)kCacheResidentSlots && !sorted_keys) {
+    if (sc.cap_max > (int64_t)kCacheResidentSlots && !ranked) {
         TraceScope ts_("msid.vote", s);
         k_ms_vote<<<kHubSamples / kThreads, kThreads, 0, s>>>(asc, n, sc.table_vals, sc.ctl);
     }
@@ -750,7 +750,7 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
     // route (a), unless the table always fits the cache; each kernel returns
     // at once on route (b).  The chunks cover
     // the largest table; those past the one in use are empty.
-    if (sc.cap_max > (int64_t)kCacheResidentSlots && !sorted_keys) {
+    if (sc.cap_max > (int64_t)kCacheResidentSlots && !ranked) {
         const int64_t nchunks = chunks_for(sc.cap_max);
         uint32_t* occ = sc.chunk;
         uint32_t* occ_before = sc.chunk + nchunks;
@@ -788,7 +788,7 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
         }
         a.vals = sc.table_vals;
         a.npass = std::max(1, (2 * sh + 7) / 8);
-        a.keep_keys = sorted_keys ? 1 : 0;
+        a.keep_keys = ranked ? 1 : 0;
         a.scratch = sc.sort.ord_cnt;
         a.status = status;
         static int configured_dev = -1;
@@ -805,7 +805,10 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
             const int rr = coop_launch(k_ms_pairs, blocks, kCoopThreads, sizeof(PairSmem), s, a);
             if (rr) return rr;
         }
-        if (sorted_keys) *sorted_keys = sc.ukeys[a.npass & 1];
+        if (ranked) {
+            *ranked = MsRanked{sc.ukeys[a.npass & 1], sc.table_vals};
+            return MSC_OK;
+        }
     }
     {
         TraceScope ts_("msid.lookup", s);

@@ -25,14 +25,19 @@ int ms_pair_shift(int64_t n);
 void size_ms_scratch(Sizer& s, int64_t n);
 MsScratch carve_ms_scratch(Carver& c, int64_t n);
 
+struct MsRanked {
+    const unsigned long long* keys;  // the K distinct pair keys (asc << ms_pair_shift(n)) | desc, ascending (K = ctl[3])
+    const uint32_t* rank_of_slot;    // rank of the pair in a table slot
+};
+
 // ms[v] = rank of (asc[v], desc[v]) among the distinct pairs, num_cells = K.
 // When `counts_known` is false the labels are validated (in range, every
 // label labels itself) and the extrema counted first; otherwise ctl[0..1]
 // must already hold the number of minima and maxima, the other control words 0.
-// `sorted_keys` (optional) receives the device array of the K distinct
-// pair keys (asc << ms_pair_shift(n)) | desc in ascending order (K = ctl[3]).
+// `ranked` (optional): ms keeps each vertex's table slot, num_cells is not
+// written, and *ranked receives what a caller needs to finish.
 int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, int32_t* num_cells,
               const MsScratch& sc, bool counts_known, int32_t* status, cudaStream_t s,
-              const unsigned long long** sorted_keys = nullptr);
+              MsRanked* ranked = nullptr);
 
 }  // namespace msc
