@@ -673,12 +673,17 @@ __global__ void __launch_bounds__(kCoopThreads) k_ord_coop(const CoopOrderArgs a
     if (nan) record_error(a.status, MSC_ERR_NAN);
 }
 
-// Largest field sorted by k_ord_coop: with two tiles per block the passes
-// lose more by their double reading than the launches cost (2^21 vertices:
-// 135 us against 179 as launches; 3 * 10^6: 200 against 176).  Eight keys per
-// thread while that leaves one tile per block at two blocks per SM (262 144:
-// 48 us, 61 with sixteen; 10^6: 93 and 76).
-constexpr int64_t kOrderCoopMax = 1 << 21;
+// Tile size of k_ord_coop for n vertices, 0 for a sort by launches.  The
+// cooperative sort is the better one while every block holds one tile
+// (loaded and ranked once) at two blocks per SM: 10^6 vertices 76 us against
+// 116 as launches (86 replayed), 1.24 * 10^6 79 against 116 (89); with two
+// tiles per block 1.5 * 10^6 take 131 against 116 (89).  Eight keys per thread
+// as long as they fit: 262 144 vertices 46 us, 61 with sixteen.
+int coop_tile(int64_t n) {
+    const int64_t blocks = 2 * (int64_t)current_device().sms;
+    if (n <= blocks * CoopSmem<uint32_t, 8>::kTile) return CoopSmem<uint32_t, 8>::kTile;
+    return n <= blocks * CoopSmem<uint32_t, 16>::kTile ? CoopSmem<uint32_t, 16>::kTile : 0;
+}
 static_assert(kCoopScratchWords + 1 <= kOrderCntWords, "the barrier word follows the counts");
 
 template <int ITEMS>
@@ -702,14 +707,14 @@ int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
 int run_order(const float* f, int64_t n, int32_t* order, uint32_t* key_a, int32_t* id_a, uint32_t* key_b,
               int32_t* id_b, const SortScratch& sc, int32_t* status, cudaStream_t s, uint32_t* barrier) {
     if (n <= 0) return MSC_OK;
-    if (n <= kOrderCoopMax) {
+    if (const int tile = coop_tile(n)) {
         if (!barrier) {
             barrier = sc.ord_cnt + kCoopScratchWords;
             MSC_TRY(cudaMemsetAsync(barrier, 0, sizeof(uint32_t), s));
         }
         const CoopOrderArgs a{f, (uint32_t)n, order, {key_a, key_b},
                               {reinterpret_cast<uint32_t*>(id_a), reinterpret_cast<uint32_t*>(id_b)}, sc.ord_cnt, barrier, status};
-        return ceil_div(n, CoopSmem<uint32_t, 8>::kTile) <= 2 * current_device().sms ? launch_coop<8>(a, s) : launch_coop<16>(a, s);
+        return tile == CoopSmem<uint32_t, 8>::kTile ? launch_coop<8>(a, s) : launch_coop<16>(a, s);
     }
     Range rg;
     rg.n = n;
