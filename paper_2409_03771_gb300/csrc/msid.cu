@@ -41,7 +41,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr unsigned long long kEmpty = ~0ull;
-constexpr uint32_t kSpread = 64;  // random spread of a pair around its home slot
+constexpr uint32_t kSpread = 64;  // random spread of a pair around its home slot (six bits of a hash)
 constexpr uint32_t kCacheResidentSlots = 1u << 20;  // 8 MiB of keys: plain random hashing
 constexpr uint32_t kPad = 4096;   // slots past the capacity: probing never wraps
 constexpr int kChunkLog2 = 12;    // route (a): chunks of 4096 slots (bases)
@@ -168,12 +168,18 @@ __device__ __forceinline__ uint32_t slot_base(uint32_t asc, unsigned long long f
 // `both`, proportional to the mean of its two extrema's ids instead: as
 // near to the vertex where both extrema are, and the many pairs of one
 // far-reaching extremum spread out with their other ends.
-__device__ __forceinline__ uint32_t home_slot(uint32_t asc, uint32_t desc, unsigned long long key, uint32_t cap,
-                                              unsigned long long f, bool both) {
-    if (cap <= kCacheResidentSlots) return (uint32_t)mix64(key) & (cap - 1);  // fits in cache: spread
+__device__ __forceinline__ uint32_t home_slot(uint32_t asc, uint32_t desc, uint32_t cap, unsigned long long f, bool both) {
+    // 32-bit hashes: a 64-bit finaliser was a quarter of the insert's instructions
+    const uint32_t hd = desc * 0x9E3779B1u;
+    if (cap <= kCacheResidentSlots) {  // fits in cache: spread
+        uint32_t h = (hd ^ asc) * 0x85EBCA77u;
+        h ^= h >> 16;
+        h = h * 0xC2B2AE3Du;
+        return (h >> 8) & (cap - 1);
+    }
     // a base is below cap for labels in [0, n); labels outside (already
     // reported) must not leave the table either
-    return min(slot_base(both ? (asc + desc) >> 1 : asc, f), cap) + (uint32_t)(mix64(key) & (kSpread - 1));
+    return min(slot_base(both ? (asc + desc) >> 1 : asc, f), cap) + (hd >> 26);
 }
 
 // Linear probing over the cap + kPad slots; `fresh` when this call stored
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
         for (int j = 0; j < kInsJ; ++j) {
             slot[j] = 0;
             if (probing >> j & 1u) {
-                h[j] = home_slot(a[j], (uint32_t)key[j] & dmask, key[j], cap, f, both);
+                h[j] = home_slot(a[j], (uint32_t)key[j] & dmask, cap, f, both);
                 w[j] = keys[h[j]];
             }
         }
