@@ -34,7 +34,6 @@ __device__ uint32_t g_sort_dbg[16];
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kItems = kSortTile / kThreads;  // 16
 constexpr int kWarps = kThreads / kWarp;      // 8
 constexpr int kBins = 256;
 constexpr unsigned long long kFlagAgg = 1ull << 62;
@@ -185,10 +184,16 @@ struct PassArgs {
     int seg_stride;
 };
 
+// Keys per thread: 64-bit sorts take 24 at two blocks per SM (six passes over
+// 52M keys and six over 14M with a payload: 2.69 ms, 2.84 with 16 at three);
+// segmented ones take the sort tile that their histograms are made by.
+template <typename KeyT>
+constexpr int kPassItems = sizeof(KeyT) == 8 ? 24 : kSortTile / kThreads;
+
 template <typename KeyT, bool VALS>
 constexpr size_t pass_smem_bytes() {
     return (size_t)(2 * kWarps * kBins + 4 * kBins + 32 + 2 * kMaxBuckets) * 4 +
-           (size_t)kSortTile * (sizeof(KeyT) + (VALS ? 4 : 0));
+           (size_t)kThreads * kPassItems<KeyT> * (sizeof(KeyT) + (VALS ? 4 : 0));
 }
 
 // One onesweep digit pass (64-bit keys alone, 52M of them: 0.40 -> 0.34 ms with
@@ -206,7 +211,10 @@ constexpr size_t pass_smem_bytes() {
 //
 // VALS: with a payload; without, keys alone are moved.
 template <typename KeyT, bool FROM_F, bool BUCKET, bool SEG, bool VALS>
-__global__ void __launch_bounds__(kThreads, 3) k_onesweep(const PassArgs<KeyT> a) {
+__global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_onesweep(const PassArgs<KeyT> a) {
+    constexpr int kItems = kPassItems<KeyT>, kTile = kThreads * kItems;
+    static_assert(kTile >= kSortTile, "the look-back words are sized for tiles of kSortTile keys");
+    static_assert(!SEG || kTile == kSortTile, "a segment's tiles and histograms are those of its table");
     extern __shared__ __align__(16) uint8_t smem[];
     uint32_t* s_whist = reinterpret_cast<uint32_t*>(smem);  // [kWarps][256]
     uint32_t* s_match = s_whist + kWarps * kBins;          // [kWarps][256] lanes per digit, 0 between keys
@@ -217,11 +225,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_onesweep(const PassArgs<KeyT> a
     uint32_t* s_misc = s_bstart + kBins;                   // [0] tile id, [1..8] scan
     uint32_t* s_bucket = s_misc + 32;                      // [2][kMaxBuckets] counts, bases
     KeyT* s_keys = reinterpret_cast<KeyT*>(s_bucket + 2 * kMaxBuckets);
-    int32_t* s_vals = reinterpret_cast<int32_t*>(s_keys + kSortTile);
+    int32_t* s_vals = reinterpret_cast<int32_t*>(s_keys + kTile);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n_all = a.d_n ? min((int64_t)*a.d_n, a.n) : a.n;  // a device count never exceeds the buffers
-    const int64_t ntiles = SEG ? a.seg_tiles : (n_all + kSortTile - 1) / kSortTile;
+    const int64_t ntiles = SEG ? a.seg_tiles : (n_all + kTile - 1) / kTile;
     if constexpr (!SEG) {
         const uint32_t c = a.hist[tid];
         s_bstart[tid] = block_scan_256(c, s_misc + 1) - c;
@@ -244,8 +252,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_onesweep(const PassArgs<KeyT> a
         }
         // tile-local 32-bit indices from here on: the tile's keys are
         // [tbase, tbase + cnt) of the packed arrays
-        const int64_t tbase = seg_base + ltile * kSortTile;
-        const int cnt = (int)min((int64_t)kSortTile, n - ltile * kSortTile);
+        const int64_t tbase = seg_base + ltile * kTile;
+        const int cnt = (int)min((int64_t)kTile, n - ltile * kTile);
         const int wbase = warp * (kItems * 32) + lane;
 
         KeyT key[kItems];
@@ -341,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_onesweep(const PassArgs<KeyT> a
                 if (d < 256u) {
                     const uint32_t lpos = s_excl[d] + s_whist[warp * kBins + d] + (rk[k] & 0xffffu);
 #ifdef MSC_DEBUG_BOUNDS
-                    if (lpos >= (uint32_t)kSortTile && atomicCAS(&g_sort_dbg[0], 0u, 1u) == 0u) {
+                    if (lpos >= (uint32_t)kTile && atomicCAS(&g_sort_dbg[0], 0u, 1u) == 0u) {
                         g_sort_dbg[1] = (uint32_t)tile; g_sort_dbg[2] = warp; g_sort_dbg[3] = lane;
                         g_sort_dbg[4] = k; g_sort_dbg[5] = d; g_sort_dbg[6] = s_excl[d];
                         g_sort_dbg[7] = s_whist[warp * kBins + d]; g_sort_dbg[8] = rk[k] & 0xffffu;
@@ -349,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_onesweep(const PassArgs<KeyT> a
                         g_sort_dbg[12] = (uint32_t)ntiles; g_sort_dbg[13] = gridDim.x;
                     }
 #endif
-                    MSC_GUARD(lpos < (uint32_t)kSortTile, a.status, -103) {
+                    MSC_GUARD(lpos < (uint32_t)kTile, a.status, -103) {
                         s_keys[lpos] = key[k];
                         if constexpr (VALS) s_vals[lpos] = val[k];
                     }
@@ -456,7 +464,7 @@ int launch_pass(const PassArgs<KeyT>& a, int64_t max_n, cudaStream_t s, const ch
     }
     int occ = 0;
     MSC_TRY(max_blocks_per_sm(&occ, kern, kThreads, smem));
-    const int64_t ntiles = SEG ? a.seg_tiles : ceil_div(max_n, kSortTile);
+    const int64_t ntiles = SEG ? a.seg_tiles : ceil_div(max_n, kThreads * kPassItems<KeyT>);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)current_device().sms * std::max(occ, 1)));
     {
         TraceScope ts_(label, s);
