@@ -259,10 +259,11 @@ int coop_blocks(K kernel, int threads, size_t smem, int64_t want, int* out) {
     return MSC_OK;
 }
 
+// The kernels here run on any number of blocks: a grid that does not fit (a
+// context confined to a part of the SMs) is halved until it does.
 template <typename... P, typename... A>
-int coop_launch(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t s, A&&... args) {
+int coop_launch(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t s, const A&... args) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -271,8 +272,13 @@ int coop_launch(void (*kernel)(P...), int blocks, int threads, size_t smem, cuda
     at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    MSC_TRY(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
-    return MSC_OK;
+    for (;; blocks /= 2) {
+        cfg.gridDim = dim3((unsigned)blocks);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+        if (e == cudaSuccess) return MSC_OK;
+        cudaGetLastError();
+        if (e != cudaErrorCooperativeLaunchTooLarge || blocks <= 1) return MSC_ERR_CUDA;
+    }
 }
 
 }  // namespace msc
