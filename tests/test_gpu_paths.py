@@ -225,6 +225,26 @@ def test_ms_id_pair_counts(m, n, roots):
     np.testing.assert_array_equal(host(ms), want)
 
 
+# 513, 1025, 2049 and 16385 chunks of slots: groups of the chunk scan that are
+# nearly empty, whole, and several per warp
+@pytest.mark.parametrize("n", [(1 << 19) + 1, 1 << 21, (1 << 21) + 3, 1 << 25])
+def test_ms_id_many_chunks(m, n):
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    lab = []
+    for _ in range(2):
+        root = torch.rand(n, device="cuda", generator=gen) < 0.3
+        ids = root.nonzero().ravel()
+        x = ids[torch.randint(ids.numel(), (n,), device="cuda", generator=gen)]
+        x[ids] = ids
+        lab.append(x.to(torch.int32))
+    keys, want = torch.unique(lab[0].long() * n + lab[1].long(), return_inverse=True)
+    ms, k = m.ms_id(*lab)
+    assert k == keys.numel()
+    assert torch.equal(ms.long(), want)
+
+
 @pytest.mark.parametrize("n", [5000, 300000, (1 << 21) + 4099, (1 << 24) + 12345])
 @pytest.mark.parametrize("bytes_", [(), (0,), (1,), (2,), (3,), (0, 2), (1, 3), (2, 3), (0, 1, 2)])
 def test_order_constant_bytes(m, n, bytes_):
