@@ -19,7 +19,9 @@
  *  - Errors found on the device are written to the caller's device status
  *    word `d_status` (int32): the call first resets it to MSC_OK, then the
  *    first error found wins (MSC_ERR_NAN, MSC_ERR_NOT_CONVERGED, MSC_ERR_ARG
- *    for an out-of-range pointer or CSR column, MSC_ERR_INTERNAL).  Read it
+ *    for an out-of-range pointer or CSR column, MSC_ERR_INTERNAL), except
+ *    that a wait inside the library that ran out replaces it with
+ *    MSC_ERR_INTERNAL and the call's later stages do no more work.  Read it
  *    after synchronising the stream.  Outputs are unspecified when it is
  *    not MSC_OK.  No device error traps or hangs the GPU: every device loop
  *    is bounded.

@@ -456,8 +456,9 @@ __global__ void __launch_bounds__(kThreads) k_adj_write(const unsigned long long
                                                         const uint32_t* __restrict__ chunk_base, int shift,
                                                         int32_t* out_a, int32_t* out_b, int64_t out_cap,
                                                         const int32_t* __restrict__ cross, const int32_t* __restrict__ order,
-                                                        int sense, unsigned long long* best) {
+                                                        int sense, unsigned long long* best, const int32_t* status) {
     __shared__ uint32_t s_w[kThreads / 32];
+    if (stage_gave_up_block(status)) return;  // the crossing vertices are indices
     const int64_t m = clamp_count(d_count, cap);
     const int64_t nchunks = (m + kChunk - 1) / kChunk;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -610,7 +611,7 @@ int finish_pairs(const PairScratch& p, int shift, int32_t* out_a, int32_t* out_b
         {
             TraceScope ts_("adjacency.write", s);
             k_adj_write<true><<<grid, kThreads, 0, s>>>(sorted, p.ctl, cap, p.chunk, shift, out_a, out_b, out_cap,
-                                                        cross, order, sense, best);
+                                                        cross, order, sense, best, status);
         }
         MSC_LAUNCHED();
         {
@@ -623,7 +624,7 @@ int finish_pairs(const PairScratch& p, int shift, int32_t* out_a, int32_t* out_b
         {
             TraceScope ts_("adjacency.write", s);
             k_adj_write<false><<<grid, kThreads, 0, s>>>(sorted, p.ctl, cap, p.chunk, shift, out_a, out_b, out_cap,
-                                                         nullptr, nullptr, 0, nullptr);
+                                                         nullptr, nullptr, 0, nullptr, status);
         }
         MSC_LAUNCHED();
     }

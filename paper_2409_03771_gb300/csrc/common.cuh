@@ -11,9 +11,27 @@ namespace msc {
 constexpr int kWarp = 32;
 
 // ----------------------------------------------------------------------------
-// device status word: the first error recorded wins
+// device status word: the first error recorded wins, except that a wait that
+// ran out (record_give_up) replaces any other
 __device__ __forceinline__ void record_error(int32_t* status, int32_t code) {
     if (status) atomicCAS(status, MSC_OK, code);
+}
+
+// A bounded wait (grid barrier, look-back, bulk copy) that ran out leaves its
+// stage's outputs unfinished: indices in them may be anything.  The call's
+// later stages are already enqueued, so those that use such an index without
+// a test of their own look here first and leave their work undone.
+__device__ __forceinline__ void record_give_up(int32_t* status) {
+    if (status) atomicExch(status, MSC_ERR_INTERNAL);
+}
+
+__device__ __forceinline__ bool stage_gave_up(const int32_t* status) {
+    return status && __ldca(status) == MSC_ERR_INTERNAL;  // written by an earlier kernel: one L2 read per SM
+}
+
+// The same for every thread of the block (kernels with barriers of their own).
+__device__ __forceinline__ bool stage_gave_up_block(const int32_t* status) {
+    return __syncthreads_or(threadIdx.x == 0 && stage_gave_up(status)) != 0;
 }
 
 // Debug builds (-DMSC_DEBUG_BOUNDS) check data-dependent addresses before

@@ -68,7 +68,9 @@ constexpr int kChunkV = kThreads * kPerThread;
 //
 // CHECKED = false (pointers made by the stencil kernels: in range and
 // acyclic by construction, since order strictly increases along them)
-// drops the per-hop range and cycle tests, and those for ended chains too.
+// drops the per-hop range and cycle tests, and those for ended chains too;
+// the kernels do nothing once a stage before them has given up a wait, which
+// may leave pointers that are neither.
 // Bound: the L1's lines per gather (LSU 65 to 80 %), no longer the
 // instructions (70 per vertex and sweep before, 40 now): a 512^3 smooth field
 // 2.43 -> 2.24 ms, white noise 1.09 -> 1.08.  Three hops per sweep take 2.61 ms
@@ -249,6 +251,7 @@ __device__ __forceinline__ uint32_t jump_sweep(const JumpPair& pr, int which, in
 
 template <bool CHECKED>
 __global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, uint32_t build_max, int32_t* status) {
+    if (!CHECKED && stage_gave_up_block(status)) return;
     jump_sweep<CHECKED>(pr, blockIdx.y, step, build_max, status);
 }
 
@@ -259,6 +262,7 @@ __global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, 
 template <bool CHECKED>
 __global__ void __launch_bounds__(kThreads) k_jump_tail(const JumpPair pr, int count, int first, int steps,
                                                         uint32_t build_max, uint32_t* barrier, int32_t* status) {
+    if (!CHECKED && stage_gave_up_block(status)) return;  // before the first barrier: every block leaves or its wait runs out
     GridBarrier bar{barrier, gridDim.x, 0};
     for (int step = first; step < steps; ++step) {
         uint32_t prev = 0;

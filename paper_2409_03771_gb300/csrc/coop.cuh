@@ -54,7 +54,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier& g, int32_t* status) {
             if (i > 64) __nanosleep(32);
         }
         s_ok = i < kBarrierLimit;
-        if (!s_ok) record_error(status, MSC_ERR_INTERNAL);
+        if (!s_ok) record_give_up(status);
         __threadfence();
     }
     __syncthreads();

@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
                                                         const int32_t* __restrict__ desc, int32_t n,
                                                         unsigned long long* keys, uint32_t* ctl, int32_t* ms,
                                                         int32_t* status) {
+    if (stage_gave_up_block(status)) return;  // the counts of extrema do not bound the pairs
     const uint32_t cap = ctl[2];
     const uint32_t lim = cap + kPad;
     const int sh = (int)ctl[kCtlShift];
@@ -672,8 +673,9 @@ __global__ void __launch_bounds__(kCoopThreads) k_ms_pairs(const PairArgs a) {
 constexpr int kLookupPer = 8;
 
 __global__ void __launch_bounds__(kThreads) k_ms_lookup(int32_t* ms, int32_t n, const uint32_t* __restrict__ vals,
-                                                        const uint32_t* ctl, int32_t* num_cells) {
+                                                        const uint32_t* ctl, int32_t* num_cells, const int32_t* status) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *num_cells = (int32_t)ctl[3];
+    if (stage_gave_up(status)) return;  // ms may hold no slots
     constexpr int64_t kChunk = (int64_t)kThreads * kLookupPer;
     for (int64_t c = blockIdx.x; c * kChunk < n; c += gridDim.x) {
         uint32_t s[kLookupPer];
@@ -837,7 +839,7 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
     }
     {
         TraceScope ts_("msid.lookup", s);
-        k_ms_lookup<<<grid_for(n / kLookupPer + 1), kThreads, 0, s>>>(ms, n, sc.table_vals, sc.ctl, num_cells);
+        k_ms_lookup<<<grid_for(n / kLookupPer + 1), kThreads, 0, s>>>(ms, n, sc.table_vals, sc.ctl, num_cells, status);
     }
     MSC_LAUNCHED();
     return MSC_OK;

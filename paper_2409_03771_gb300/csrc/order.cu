@@ -311,6 +311,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     constexpr bool FF = SHIFT == 0;
     uint32_t* keys_out = key_of(a.bufs, to);  // kOutBuckets: the positions of the filed pairs
     int32_t* vals_out = id_of(a.bufs, to);    // ... and their ids
+    if (SHIFT > 0 && stage_gave_up_block(a.status)) return;  // the ids of an unfinished pass
     // few populated digits in this pass (a float field's top byte): rank
     // with match
     const bool use_match = __syncthreads_count(a.total[tid] != 0u) <= MSC_ORD_MATCH_MAX;
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
             if (__syncthreads_or(!ok)) {
                 // a copy never landed: report, let the prefetch in flight finish, stop
                 if (tid == 0) {
-                    record_error(a.status, MSC_ERR_INTERNAL);
+                    record_give_up(a.status);
                     if (tn >= 0 && by_tma(tn)) mbar_wait(&mbar[slot ^ 1], (uint32_t)((it + 1) >> 1) & 1u, kWaitLimit);
                 }
                 return;

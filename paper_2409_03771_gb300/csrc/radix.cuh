@@ -152,6 +152,7 @@ __device__ __forceinline__ void permute_pairs(const int32_t* __restrict__ ids, c
                                               bool vec, int32_t* __restrict__ order, int32_t* status) {
     const int64_t c0 = (int64_t)blockIdx.x * kPermuteChunk + 4 * threadIdx.x;
     int4 id[kPermutePer], p[kPermutePer];
+    const bool unfinished = stage_gave_up(status);  // in flight with the pairs
 #pragma unroll
     for (int q = 0; q < kPermutePer; ++q) {
         const int64_t i = c0 + q * (4 * kPermuteThreads);
@@ -160,6 +161,7 @@ __device__ __forceinline__ void permute_pairs(const int32_t* __restrict__ ids, c
             p[q] = __ldcs(reinterpret_cast<const int4*>(pos + i));
         }
     }
+    if (unfinished) return;
 #pragma unroll
     for (int q = 0; q < kPermutePer; ++q) {
         const int64_t i = c0 + q * (4 * kPermuteThreads);

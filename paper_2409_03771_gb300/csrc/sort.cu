@@ -230,6 +230,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_oneswee
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n_all = a.d_n ? min((int64_t)*a.d_n, a.n) : a.n;  // a device count never exceeds the buffers
     const int64_t ntiles = SEG ? a.seg_tiles : (n_all + kTile - 1) / kTile;
+    if (stage_gave_up_block(a.status)) return;  // an earlier pass: the payloads are indices
     if constexpr (!SEG) {
         const uint32_t c = a.hist[tid];
         s_bstart[tid] = block_scan_256(c, s_misc + 1) - c;
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_oneswee
                     const unsigned long long flag = w & (3ull << 62);
                     if (wep != a.epoch || flag == 0) {
                         if (++spins > kSpinLimit) {
-                            record_error(a.status, MSC_ERR_INTERNAL);
+                            record_give_up(a.status);
                             break;
                         }
                         __nanosleep(32);

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_steepest_tma(const __grid_const
         // one barrier per tile: the buffer is free again, and a failed wait
         // (never expected) is seen by every thread
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) record_error(status, MSC_ERR_INTERNAL);
+            if (tid == 0) record_give_up(status);
             for (int q = 0; q < kStages; ++q) mbar_wait(&bar[q], phase[q], kWaitLimit);
             return;
         }
