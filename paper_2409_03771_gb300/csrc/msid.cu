@@ -183,34 +183,48 @@ __device__ __forceinline__ uint32_t home_slot(uint32_t asc, uint32_t desc, uint3
 }
 
 // Linear probing over the cap + kPad slots; `fresh` when this call stored
-// the key.  Probe i looks at slot home + i; after kNearProbes slots it goes
-// on from a second, random home, so that the many pairs of one minimum (all
-// with one home window) cannot build one long cluster.  Every insert of a
-// key follows the same sequence, so equal keys meet.  Leaving the home
+// the key.  Probe i looks at slot home + i; after kNear slots it goes on from
+// a second, random home, so that the many pairs of one minimum (all with one
+// home window) cannot build one long cluster.  Homes by both labels (BOTH)
+// need more: means of two labels crowd around the middle of the table where
+// the labels have no order in space, fill it solidly, and a walk on from a
+// random place inside such a part is as long as the part (8.4M vertices of
+// random labels, 30 % of them with one minimum: 14 s; 9.7 ms with homes by the
+// minimum).  There the probe tries kFarProbes slots from each of kFarHomes
+// random homes before it walks the table (2.6 ms), and leaves its first home
+// after kNearBoth slots, as nothing depends on where a pair lands (128: a third
+// slower there, no difference on fields).  Every insert of a key follows the
+// same sequence, so equal keys meet.  Leaving the home
 // window or running off the end (the probe then continues at slot 0) sets
 // `broke`: a pair is no longer within M of its base.  The probe resumes at
 // step i0 (slot h0), after the steps a caller made itself.
 constexpr uint32_t kNearProbes = 1024;
+constexpr uint32_t kNearBoth = 32;
+constexpr uint32_t kFarProbes = 16;
+constexpr uint32_t kFarHomes = 64;
 static_assert(kPad % 4 == 0, "the table's slot count is a multiple of four");
 
+template <bool BOTH>
 __device__ __forceinline__ uint32_t probe_insert(unsigned long long* keys, uint32_t cap, unsigned long long key,
                                                  uint32_t i0, uint32_t h0, bool& fresh, bool& broke,
                                                  int32_t* status) {
+    constexpr uint32_t kNear = BOTH ? kNearBoth : kNearProbes;
+    constexpr uint32_t kFar = kNear + (BOTH ? kFarHomes * kFarProbes : 0);  // from here on one walk
     const uint32_t lim = cap + kPad;
     uint32_t h = h0;
     // One round trip reads the aligned group of four slots (one 32-byte
     // sector) holding slot h and takes the first of slots h, h+1, ... in it
-    // that holds the key or is empty.  The steps stop exactly at kNearProbes
-    // and at the end of the table (lim, a multiple of four), so every insert
-    // of a key visits the same slots in the same order.
-    uint32_t i = i0;
-    while (i < lim + kNearProbes) {
-        if (i == kNearProbes) {
-            h = (uint32_t)mix64(key ^ 0x9e3779b97f4a7c15ull) & (cap - 1);
+    // that holds the key or is empty.  The steps stop exactly at `next` (the
+    // next random home) and at the end of the table (lim, a multiple of four),
+    // so every insert of a key visits the same slots in the same order.
+    uint32_t i = i0, next = kNear;
+    while (i < lim + kFar) {
+        if (i == next) {
+            h = (uint32_t)mix64(key + i * 0x9e3779b97f4a7c15ull) & (cap - 1);
+            next = i < kFar ? i + kFarProbes : ~0u;
             broke = true;
         }
-        const uint32_t g0 = h & ~3u, start = h - g0;
-        const uint32_t end = i < kNearProbes ? min(4u, start + (kNearProbes - i)) : 4u;
+        const uint32_t g0 = h & ~3u, start = h - g0, end = min(4u, start + (next - i));
         const ulonglong2 lo = *reinterpret_cast<const ulonglong2*>(keys + g0);
         const ulonglong2 hi = *reinterpret_cast<const ulonglong2*>(keys + g0 + 2);
         const unsigned long long sl[4] = {lo.x, lo.y, hi.x, hi.y};
@@ -243,7 +257,7 @@ __device__ __forceinline__ uint32_t probe_insert(unsigned long long* keys, uint3
             broke = true;
         }
     }
-    record_error(status, MSC_ERR_INTERNAL);  // table full: impossible at load <= 1/2
+    record_error(status, MSC_ERR_INTERNAL);  // no slot free: there are more slots than distinct pairs
     return 0;
 }
 
@@ -255,18 +269,13 @@ __device__ __forceinline__ uint32_t probe_insert(unsigned long long* keys, uint3
 #endif
 constexpr int kInsJ = MSC_MS_INSERT_J;
 
-__global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restrict__ asc,
-                                                        const int32_t* __restrict__ desc, int32_t n,
-                                                        unsigned long long* keys, uint32_t* ctl, int32_t* ms,
-                                                        int32_t* status) {
-    if (stage_gave_up_block(status)) return;  // the counts of extrema do not bound the pairs
+template <bool BOTH>
+__device__ __forceinline__ void insert_pairs(const int32_t* __restrict__ asc, const int32_t* __restrict__ desc, int32_t n,
+                                             unsigned long long* keys, uint32_t* ctl, int32_t* ms, int32_t* status) {
     const uint32_t cap = ctl[2];
     const uint32_t lim = cap + kPad;
     const int sh = (int)ctl[kCtlShift];
-    // fixed before this kernel starts (ctl[kCtlRoute] changes while it runs):
-    // every insert of a key has to follow the same probes
-    const bool both = ctl[kCtlHome] != 0u;
-    const bool ordered = cap > kCacheResidentSlots && !both;
+    const bool ordered = cap > kCacheResidentSlots && !BOTH;
     const unsigned long long f = (unsigned long long)ctl[9] | ((unsigned long long)ctl[10] << 32);
     const uint32_t dmask = (1u << sh) - 1u;  // sh = ceil(log2 n) <= 31
     const int lane = threadIdx.x & 31;
@@ -298,7 +307,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
         for (int j = 0; j < kInsJ; ++j) {
             slot[j] = 0;
             if (probing >> j & 1u) {
-                h[j] = home_slot(a[j], (uint32_t)key[j] & dmask, cap, f, both);
+                h[j] = home_slot(a[j], (uint32_t)key[j] & dmask, cap, f, BOTH);
                 w[j] = keys[h[j]];
             }
         }
@@ -320,7 +329,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
                     h1 = 0;
                     broke = true;
                 }
-                slot[j] = probe_insert(keys, cap, key[j], 1, h1, fresh, broke, status);
+                slot[j] = probe_insert<BOTH>(keys, cap, key[j], 1, h1, fresh, broke, status);
             }
             added += fresh;
             // how far past its base a pair landed (route (a))
@@ -341,6 +350,17 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
         if (added) atomicAdd(&ctl[3], added);
         if (far) atomicMax(&ctl[kCtlM], far);
     }
+}
+
+__global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restrict__ asc,
+                                                        const int32_t* __restrict__ desc, int32_t n,
+                                                        unsigned long long* keys, uint32_t* ctl, int32_t* ms,
+                                                        int32_t* status) {
+    if (stage_gave_up_block(status)) return;  // the counts of extrema do not bound the pairs
+    // fixed before this kernel starts (ctl[kCtlRoute] changes while it runs):
+    // every insert of a key has to follow the same probes
+    if (ctl[kCtlHome] != 0u) insert_pairs<true>(asc, desc, n, keys, ctl, ms, status);
+    else insert_pairs<false>(asc, desc, n, keys, ctl, ms, status);
 }
 
 // Route (a), step 1: occupied slots per chunk of slots.

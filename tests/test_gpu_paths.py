@@ -280,3 +280,53 @@ def test_adjacency_key_counts(m, oracle_mod, dims, bound, conn):
     got = m.adjacency_grid(cuda(lab), dims, conn, label_bound=bound)
     for g, w in zip(got, oracle_mod.adjacency_grid(lab, dims, conn)):
         np.testing.assert_array_equal(host(g), w)
+
+
+# ---------------------------------------------------------------------------
+# cell ids of labels without an order in space, with an extremum that holds
+# very many vertices: the homes by both labels crowd in one part of the table
+
+
+def spread_labels(kind, n, gen):
+    """Minimum and maximum labels that label themselves."""
+    def roots(share):
+        return (torch.rand(n, device="cuda", generator=gen) < share).nonzero().ravel()
+
+    def pick(ids):
+        lab = ids[torch.randint(ids.numel(), (n,), device="cuda", generator=gen)]
+        lab[ids] = ids
+        return lab
+
+    if kind == "mirrored":  # desc = n - 1 - asc: one mean for all pairs
+        half = (torch.rand(n // 2, device="cuda", generator=gen) < 0.3).nonzero().ravel()
+        ids = torch.cat([half, n - 1 - half])
+        asc = pick(ids)
+        desc = n - 1 - asc
+        desc[ids] = ids
+    else:
+        share = 0.3 if kind == "random" else 3000 / n
+        ids = roots(share)
+        asc, desc = pick(ids), pick(roots(share))
+    hub = torch.rand(n, device="cuda", generator=gen) < 0.3
+    keep = asc == torch.arange(n, device="cuda")
+    asc = torch.where(hub & ~keep, ids[-1], asc)
+    return asc.int(), desc.int()
+
+
+@pytest.mark.parametrize("n", [(1 << 21) - 5, 1 << 21, 1 << 22])
+@pytest.mark.parametrize("kind", ["random", "few", "mirrored"])
+def test_ms_id_crowded_homes(m, kind, n):
+    asc, desc = spread_labels(kind, n, torch.Generator(device="cuda").manual_seed(n))
+    keys, want = torch.unique(asc.long() * n + desc.long(), return_inverse=True)
+    times = []
+    for _ in range(2):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        ms, k = m.ms_id(asc, desc)
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    assert k == keys.numel()
+    assert torch.equal(ms.long(), want)
+    # a walk through a part of the table that is full takes 950 ms at 2^21; homes by the minimum alone 3.7 to 12 ms
+    assert min(times) < 50.0, times
