@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(kThreads) k_batch_rebase(const int32_t* __rest
                                                            const int32_t* __restrict__ first,
                                                            const uint32_t* __restrict__ rank_of_slot, int64_t tiles,
                                                            int32_t* __restrict__ ms, int32_t* __restrict__ asc,
-                                                           int32_t* __restrict__ desc, const int32_t* status) {
-    if (stage_gave_up(status)) return;  // ms may hold no slots
+                                                           int32_t* __restrict__ desc, const uint32_t* skip) {
+    if (*skip != 0u) return;  // ms holds no slots
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int i = tile_seg[t];
         const int32_t o = off[i], n = off[i + 1] - o, fr = first[i];
@@ -369,7 +369,7 @@ int run_batch(void* ws, size_t ws_bytes, const Layout& L, const DevLayout& d, co
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(L.tiles, (int64_t)current_device().sms * 8));
         TraceScope ts_("batch.rebase", s);
         k_batch_rebase<<<grid, kThreads, 0, s>>>(d.tile_seg, d.off, d.tile0, d.first, ranked.rank_of_slot, L.tiles,
-                                                 B.ms, B.asc, B.desc, B.status);
+                                                 B.ms, B.asc, B.desc, ranked.skip);
     }
     MSC_LAUNCHED();
     return MSC_OK;

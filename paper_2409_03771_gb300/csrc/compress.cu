@@ -251,7 +251,8 @@ __device__ __forceinline__ uint32_t jump_sweep(const JumpPair& pr, int which, in
 
 template <bool CHECKED>
 __global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, uint32_t build_max, int32_t* status) {
-    if (!CHECKED && stage_gave_up_block(status)) return;
+    // (a first sweep that does nothing counts no changes, so the later ones return too)
+    if (!CHECKED && step == 0 && stage_gave_up_block(status)) return;
     jump_sweep<CHECKED>(pr, blockIdx.y, step, build_max, status);
 }
 
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kThreads) k_jump(const JumpPair pr, int step, 
 template <bool CHECKED>
 __global__ void __launch_bounds__(kThreads) k_jump_tail(const JumpPair pr, int count, int first, int steps,
                                                         uint32_t build_max, uint32_t* barrier, int32_t* status) {
-    if (!CHECKED && stage_gave_up_block(status)) return;  // before the first barrier: every block leaves or its wait runs out
+    if (!CHECKED && first == 0 && stage_gave_up_block(status)) return;  // before the first barrier: every block leaves or its wait runs out
     GridBarrier bar{barrier, gridDim.x, 0};
     for (int step = first; step < steps; ++step) {
         uint32_t prev = 0;

@@ -57,6 +57,7 @@ constexpr int kCtlM = 17;       // largest slot - asc * cap / n of a pair
 constexpr int kCtlCompact = 18; // route (b): compacted pairs
 constexpr int kCtlShift = 19;   // b of the pair keys
 constexpr int kCtlHome = 20;    // home slots of a table too big for the cache: 0 by the minimum, 1 by both labels
+constexpr int kCtlSkip = 21;    // a stage before this one gave up a wait: no pairs are inserted, ms holds no slots
 constexpr int kCtlBarrier = 40; // two grid barriers of the pair sort, zero at its start
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
@@ -116,7 +117,8 @@ constexpr uint32_t kHubVotes = 24;
 // Empties the table and the vote counters and writes the control words
 // (every block works the capacity out for itself: one launch fewer).
 __global__ void __launch_bounds__(kThreads) k_ms_clear(unsigned long long* keys, uint32_t* votes, uint32_t* ctl,
-                                                       int64_t n, int64_t cap_max, int sh, int force_sort) {
+                                                       int64_t n, int64_t cap_max, int sh, int force_sort,
+                                                       const int32_t* status) {
     const unsigned long long cap = table_capacity(ctl, n, cap_max);
     const int64_t slots = (int64_t)cap + kPad, t0 = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (t0 == 0) {
@@ -131,6 +133,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_clear(unsigned long long* keys,
         ctl[kCtlM] = 0;
         ctl[kCtlCompact] = 0;
         ctl[kCtlShift] = (uint32_t)sh;
+        ctl[kCtlSkip] = stage_gave_up(status);
     }
     for (int64_t i = t0; i < slots; i += (int64_t)gridDim.x * kThreads) keys[i] = kEmpty;
     if (cap > kCacheResidentSlots && t0 < kHubCounters) votes[t0] = 0;
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(kThreads) k_ms_insert(const int32_t* __restric
                                                         const int32_t* __restrict__ desc, int32_t n,
                                                         unsigned long long* keys, uint32_t* ctl, int32_t* ms,
                                                         int32_t* status) {
-    if (stage_gave_up_block(status)) return;  // the counts of extrema do not bound the pairs
+    if (ctl[kCtlSkip] != 0u) return;  // the counts of extrema do not bound the pairs
     // fixed before this kernel starts (ctl[kCtlRoute] changes while it runs):
     // every insert of a key has to follow the same probes
     if (ctl[kCtlHome] != 0u) insert_pairs<true>(asc, desc, n, keys, ctl, ms, status);
@@ -693,9 +696,9 @@ __global__ void __launch_bounds__(kCoopThreads) k_ms_pairs(const PairArgs a) {
 constexpr int kLookupPer = 8;
 
 __global__ void __launch_bounds__(kThreads) k_ms_lookup(int32_t* ms, int32_t n, const uint32_t* __restrict__ vals,
-                                                        const uint32_t* ctl, int32_t* num_cells, const int32_t* status) {
+                                                        const uint32_t* ctl, int32_t* num_cells) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *num_cells = (int32_t)ctl[3];
-    if (stage_gave_up(status)) return;  // ms may hold no slots
+    if (ctl[kCtlSkip] != 0u) return;
     constexpr int64_t kChunk = (int64_t)kThreads * kLookupPer;
     for (int64_t c = blockIdx.x; c * kChunk < n; c += gridDim.x) {
         uint32_t s[kLookupPer];
@@ -781,7 +784,7 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
         TraceScope ts_("msid.clear", s);
         // at least kHubCounters threads, so that every vote counter is cleared
         const int grid = std::max(grid_for(sc.cap_max + kPad, 4), kHubCounters / kThreads);
-        k_ms_clear<<<grid, kThreads, 0, s>>>(sc.table_keys, sc.table_vals, sc.ctl, n, sc.cap_max, sh, ranked ? 1 : 0);
+        k_ms_clear<<<grid, kThreads, 0, s>>>(sc.table_keys, sc.table_vals, sc.ctl, n, sc.cap_max, sh, ranked ? 1 : 0, status);
     }
     MSC_LAUNCHED();
     if (sc.cap_max > (int64_t)kCacheResidentSlots && !ranked) {
@@ -853,13 +856,13 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
             if (rr) return rr;
         }
         if (ranked) {
-            *ranked = MsRanked{sc.ukeys[a.npass & 1], sc.table_vals};
+            *ranked = MsRanked{sc.ukeys[a.npass & 1], sc.table_vals, sc.ctl + kCtlSkip};
             return MSC_OK;
         }
     }
     {
         TraceScope ts_("msid.lookup", s);
-        k_ms_lookup<<<grid_for(n / kLookupPer + 1), kThreads, 0, s>>>(ms, n, sc.table_vals, sc.ctl, num_cells, status);
+        k_ms_lookup<<<grid_for(n / kLookupPer + 1), kThreads, 0, s>>>(ms, n, sc.table_vals, sc.ctl, num_cells);
     }
     MSC_LAUNCHED();
     return MSC_OK;

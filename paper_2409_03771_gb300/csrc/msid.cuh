@@ -14,7 +14,7 @@ struct MsScratch {
     int64_t cap_max;
     unsigned long long* ukeys[2];    // [n] unique pair keys (ping-pong)
     int32_t* uvals[2];               // [n] their table slots
-    uint32_t* ctl;                   // [0] nmin [1] nmax [2] cap [3] K; words 9..20 private; words 40, 41 zero at the start
+    uint32_t* ctl;                   // [0] nmin [1] nmax [2] cap [3] K; words 9..21 private; words 40, 41 zero at the start
     uint32_t* chunk;                 // [2][chunks of 4096 minimum ids]: pair counts, their scan
     SortScratch sort;
 };
@@ -28,6 +28,7 @@ MsScratch carve_ms_scratch(Carver& c, int64_t n);
 struct MsRanked {
     const unsigned long long* keys;  // the K distinct pair keys (asc << ms_pair_shift(n)) | desc, ascending (K = ctl[3])
     const uint32_t* rank_of_slot;    // rank of the pair in a table slot
+    const uint32_t* skip;            // not 0: a stage before the cell ids gave up, ms holds no slots
 };
 
 // ms[v] = rank of (asc[v], desc[v]) among the distinct pairs, num_cells = K.

@@ -311,7 +311,6 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     constexpr bool FF = SHIFT == 0;
     uint32_t* keys_out = key_of(a.bufs, to);  // kOutBuckets: the positions of the filed pairs
     int32_t* vals_out = id_of(a.bufs, to);    // ... and their ids
-    if (SHIFT > 0 && stage_gave_up_block(a.status)) return;  // the ids of an unfinished pass
     // few populated digits in this pass (a float field's top byte): rank
     // with match
     const bool use_match = __syncthreads_count(a.total[tid] != 0u) <= MSC_ORD_MATCH_MAX;
@@ -326,12 +325,14 @@ __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownA
     for (int i = tid; i < kW * kB / 2; i += kT) reinterpret_cast<uint32_t*>(s_wh)[i] = 0u;
     for (int i = tid; i < kW * kB; i += kT) s_match[i] = 0u;
     if (tid == 0) {
+        s_misc[31] = SHIFT > 0 && stage_gave_up(a.status);
         mbar_init(&mbar[0], 1);
         mbar_init(&mbar[1], 1);
         fence_mbar_init();
     }
     __syncthreads();
 
+    if (s_misc[31]) return;  // the ids of an unfinished pass
     const uint32_t* src_k = ff ? reinterpret_cast<const uint32_t*>(a.bufs.f) : key_of(a.bufs, from);
     const int32_t* src_v = ff ? nullptr : id_of(a.bufs, from);
     const bool use_tma = ff ? a.bufs.aligned[2] : from ? a.bufs.aligned[1] : a.bufs.aligned[0];

@@ -230,14 +230,17 @@ __global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_oneswee
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n_all = a.d_n ? min((int64_t)*a.d_n, a.n) : a.n;  // a device count never exceeds the buffers
     const int64_t ntiles = SEG ? a.seg_tiles : (n_all + kTile - 1) / kTile;
-    if (stage_gave_up_block(a.status)) return;  // an earlier pass: the payloads are indices
     if constexpr (!SEG) {
         const uint32_t c = a.hist[tid];
         s_bstart[tid] = block_scan_256(c, s_misc + 1) - c;
     }
     for (int i = tid; i < kWarps * kBins; i += kThreads) s_match[i] = 0;
     for (;;) {
-        if (tid == 0) s_misc[0] = atomicAdd(a.tile_counter, 1u);
+        if (tid == 0) {  // no tiles left once a pass before this one gave up: its payloads are indices
+            const bool unfinished = stage_gave_up(a.status);
+            const uint32_t next = atomicAdd(a.tile_counter, 1u);
+            s_misc[0] = unfinished ? ~0u : next;
+        }
         for (int i = tid; i < kWarps * kBins; i += kThreads) s_whist[i] = 0;
         __syncthreads();
         const int64_t tile = s_misc[0];
