@@ -278,13 +278,19 @@ __global__ void __launch_bounds__(kThreads) k_jump_tail(const JumpPair pr, int c
 
 // Sweeps launched over the whole GPU before the tail: the ones that usually
 // have work.  All sweeps of a small array go into the tail (64^3 vertices:
-// 62 us as eleven launches, 28 as one; 256^3, four launches and the tail: 163
-// -> 127).  Large arrays keep eight launches, so that only paths of more than
-// 390 000 steps meet the tail's smaller grid.
+// 62 us as eleven launches, 28 as one).  Below 2^24 vertices four do, and
+// from there on eight: fields have nothing left to do after four or five (256 x
+// 256 x 250 noise: 159 us as thirteen launches, 122 now), but on paths of more
+// than 625 steps the tail goes on with whole sweeps.
+// The tail's grid: two blocks per SM up to 2^21 vertices (a random chain of
+// 10^6: 128 us, 157 with four) and where it has nothing left to do, which
+// leaves room to start beside other streams' kernels; four between, where
+// long paths need them (one path of 10^7 vertices: 476 us with two, 408 with
+// four, 404 as a launch per sweep; 2^24 - 1: 738, 628, 625).
 constexpr int64_t kTailVertices = 1 << 20;
 constexpr int64_t kLargeVertices = 1 << 24;
 int full_sweeps(int64_t n) { return n <= kTailVertices ? 0 : n < kLargeVertices ? 4 : 8; }
-constexpr int kTailBlocksPerSm = 2;  // leaves room to start beside other streams' kernels
+int tail_blocks_per_sm(int64_t n) { return n <= 2 * kTailVertices || n >= kLargeVertices ? 2 : 4; }
 
 }  // namespace
 
@@ -347,7 +353,7 @@ int run_compress(int32_t* const* ptrs, int count, int32_t n, const CompressScrat
     auto tail = tune.trusted ? k_jump_tail<false> : k_jump_tail<true>;
     int blocks = 0;
     const int r = coop_blocks(
-        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * kTailBlocksPerSm), &blocks);
+        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * tail_blocks_per_sm(n)), &blocks);
     if (r) return r;
     TraceScope ts_("compress.tail", s);
     return coop_launch(tail, blocks, kThreads, 0, s, pr, count, full, steps, build_max, &sc.ctl[0].barrier, status);
