@@ -351,3 +351,27 @@ def test_compress_line_costs_the_same_on_both_sides_of_the_launch_rule(m):
         assert int(st) == m.OK and int(p.max()) == 0
         best.append(min(times))
     assert best[0] < 1.12 * best[1], best  # 1.23 with a tail of two blocks per SM, 1.04 as a launch per sweep
+
+
+# (mask, 6 or 14 neighbours, stage, us per call): between what the stage takes and what it took with finds one after
+# the other and run starts from masks (1550 and 2270 us)
+@pytest.mark.parametrize("dims,kind,conn,stage,limit", [((512, 512, 512), 0.5, 6, "cc.local", 1300.0),
+                                                        ((512, 512, 512), 0.5, 14, "cc.local", 1900.0)])
+
+def test_cc_mask_stage_times(m, dims, kind, conn, stage, limit):
+    n = dims[0] * dims[1] * dims[2]
+    if kind == "checker":
+        i = torch.arange(n, device="cuda")
+        mask = ((i % dims[0] + i // dims[0] % dims[1] + i // (dims[0] * dims[1])) & 1).to(torch.uint8)
+    else:
+        mask = (torch.rand(n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1)) < kind).to(torch.uint8)
+    times = []
+    m.cc_mask(mask, dims, conn)
+    for _ in range(6):
+        m.msc_trace_reset()
+        m.msc_trace_enable(True)
+        m.cc_mask(mask, dims, conn)
+        m.msc_trace_enable(False)
+        times.append(m.msc_trace_collect()[stage][1] * 1e3)
+    m.msc_trace_reset()
+    assert min(times) < limit, times
