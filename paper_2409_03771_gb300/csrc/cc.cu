@@ -479,6 +479,68 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 4) k_cc_merge(const uint8_t*
 constexpr int kFlatBytes = 32;  // mask bytes per thread
 constexpr int kFlatChunk = kThreads * kFlatBytes;
 
+// Voxels v .. v + 3, of which some are masked.
+__device__ __forceinline__ void flatten_quad(int32_t* label, int64_t v, int64_t n, int label16) {
+    const bool whole = label16 && v + 4 <= n;
+    int32_t l[4], r[4];
+    if (whole) {
+        const int4 x = *reinterpret_cast<const int4*>(label + v);
+        l[0] = x.x, l[1] = x.y, l[2] = x.z, l[3] = x.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) l[j] = v + j < n ? label[v + j] : -1;
+    }
+    uint32_t open = 0, moved = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        r[j] = l[j];
+        open |= (l[j] >= 0 && (j == 0 || l[j] != l[j - 1]) ? 1u : 0u) << j;
+    }
+    for (uint32_t it = 0; it < kUnionLimit && open; ++it) {  // bound only: chains are short
+        int32_t up[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) up[j] = open >> j & 1u ? label[r[j]] : 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (open >> j & 1u) {
+                if (up[j] == r[j]) open &= ~(1u << j);
+                else {
+                    r[j] = up[j];
+                    moved |= 1u << j;
+                }
+            }
+    }
+    if (!moved) return;
+#pragma unroll
+    for (int j = 1; j < 4; ++j)
+        if (l[j] == l[j - 1]) r[j] = r[j - 1];
+    if (whole) {
+        *reinterpret_cast<int4*>(label + v) = make_int4(r[0], r[1], r[2], r[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (r[j] != l[j]) label[v + j] = r[j];
+    }
+}
+
+// A small mask: a quad per thread, as chunks would leave most of the GPU
+// without a block (48^3: fourteen of them).  48^3, half set: 14 -> 6 us; 128^3: 15
+// -> 9.  Beyond, dense masks gain and sparse ones lose (203 x 150 x 177, 2 %
+// set: the call 88 -> 92 us).
+constexpr int64_t kFlatSmall = 1 << 21;
+
+__global__ void __launch_bounds__(kThreads) k_cc_flatten_small(const uint8_t* __restrict__ mask, int64_t n, int mask4,
+                                                               int label16, int32_t* label) {
+    const int64_t v = 4 * ((int64_t)blockIdx.x * kThreads + threadIdx.x);
+    uint32_t any = 0;
+    if (mask4 && v + 4 <= n) {
+        any = __ldg(reinterpret_cast<const uint32_t*>(mask + v));
+    } else {
+        for (int64_t u = v; u < min(n, v + 4); ++u) any |= mask[u];
+    }
+    if (any) flatten_quad(label, v, n, label16);
+}
+
 __global__ void __launch_bounds__(kThreads) k_cc_flatten(const uint8_t* __restrict__ mask, int64_t n, int mask16, int label16,
                                                          int32_t* label) {
     __shared__ uint16_t s_quad[kFlatChunk / 4];
@@ -531,47 +593,7 @@ __global__ void __launch_bounds__(kThreads) k_cc_flatten(const uint8_t* __restri
         const uint32_t total = s_count;
         if (c0 + stride < n) load(c0 + stride, w);  // in flight while this chunk's quads are followed
         for (uint32_t i = tid; i < total; i += kThreads) {
-            const int64_t v = c0 + 4 * (int64_t)s_quad[i];
-            const bool whole = label16 && v + 4 <= n;
-            int32_t l[4], r[4];
-            if (whole) {
-                const int4 x = *reinterpret_cast<const int4*>(label + v);
-                l[0] = x.x, l[1] = x.y, l[2] = x.z, l[3] = x.w;
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) l[j] = v + j < n ? label[v + j] : -1;
-            }
-            uint32_t open = 0, moved = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                r[j] = l[j];
-                open |= (l[j] >= 0 && (j == 0 || l[j] != l[j - 1]) ? 1u : 0u) << j;
-            }
-            for (uint32_t it = 0; it < kUnionLimit && open; ++it) {  // bound only: chains are short
-                int32_t up[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) up[j] = open >> j & 1u ? label[r[j]] : 0;
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (open >> j & 1u) {
-                        if (up[j] == r[j]) open &= ~(1u << j);
-                        else {
-                            r[j] = up[j];
-                            moved |= 1u << j;
-                        }
-                    }
-            }
-            if (!moved) continue;
-#pragma unroll
-            for (int j = 1; j < 4; ++j)
-                if (l[j] == l[j - 1]) r[j] = r[j - 1];
-            if (whole) {
-                *reinterpret_cast<int4*>(label + v) = make_int4(r[0], r[1], r[2], r[3]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (r[j] != l[j]) label[v + j] = r[j];
-            }
+            flatten_quad(label, c0 + 4 * (int64_t)s_quad[i], n, label16);
         }
         __syncthreads();
     }
@@ -773,7 +795,11 @@ int run_cc_mask(const uint8_t* mask, msc_grid gd, int conn, int32_t* label, int3
     MSC_LAUNCHED();
     {
         TraceScope ts_("cc.flatten", s);
-        k_cc_flatten<<<cc_grid_for(ceil_div(g.n, kFlatBytes), 6), kThreads, 0, s>>>(
+        if (g.n <= kFlatSmall)
+            k_cc_flatten_small<<<(unsigned)ceil_div(g.n, 4 * kThreads), kThreads, 0, s>>>(
+                mask, g.n, ((uintptr_t)mask & 3) == 0, ((uintptr_t)label & 15) == 0, label);
+        else
+            k_cc_flatten<<<cc_grid_for(ceil_div(g.n, kFlatBytes), 6), kThreads, 0, s>>>(
             mask, g.n, ((uintptr_t)mask & 15) == 0, ((uintptr_t)label & 15) == 0, label);
     }
     MSC_LAUNCHED();

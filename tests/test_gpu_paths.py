@@ -353,11 +353,31 @@ def test_compress_line_costs_the_same_on_both_sides_of_the_launch_rule(m):
     assert best[0] < 1.12 * best[1], best  # 1.23 with a tail of two blocks per SM, 1.04 as a launch per sweep
 
 
-# (mask, 6 or 14 neighbours, stage, us per call): between what the stage takes and what it took with finds one after
-# the other and run starts from masks (1550 and 2270 us)
-@pytest.mark.parametrize("dims,kind,conn,stage,limit", [((512, 512, 512), 0.5, 6, "cc.local", 1300.0),
-                                                        ((512, 512, 512), 0.5, 14, "cc.local", 1900.0)])
+# ---------------------------------------------------------------------------
+# mask components: small grids (a quad of voxels per thread), noisy masks
 
+
+@pytest.mark.parametrize("conn", [6, 14])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (3, 1, 1), (5, 3, 2), (127, 129, 128), (128, 128, 128), (129, 128, 128), (131, 127, 131)])
+@pytest.mark.parametrize("density", [0.02, 0.5])
+@pytest.mark.parametrize("offset", [0, 1, 3])
+def test_cc_mask_small_grids(m, oracle_mod, conn, dims, density, offset):
+    n = dims[0] * dims[1] * dims[2]
+    mask = (np.random.default_rng(n + conn).random(n) < density).astype(np.uint8) * 7
+    buf = torch.empty(n + offset, dtype=torch.uint8, device="cuda")
+    buf[offset:] = cuda(mask)
+    lab = torch.empty(n + offset, dtype=torch.int32, device="cuda")[offset:]
+    ws, st = torch.empty(256, dtype=torch.uint8, device="cuda"), torch.empty(1, dtype=torch.int32, device="cuda")
+    assert m.msc_cc_mask(buf[offset:], dims, conn, lab, ws, ws.numel(), st) == m.OK
+    assert int(st) == m.OK
+    np.testing.assert_array_equal(host(lab), oracle_mod.cc_grid(mask, dims, conn))
+
+
+# (mask, 6 or 14 neighbours, stage, us per call): between what the stage takes and what it took with finds one after
+# the other and run starts from masks (1550 and 2270 us) or in chunks of 8192 voxels (14 us)
+@pytest.mark.parametrize("dims,kind,conn,stage,limit", [((512, 512, 512), 0.5, 6, "cc.local", 1300.0),
+                                                        ((512, 512, 512), 0.5, 14, "cc.local", 1900.0),
+                                                        ((48, 48, 48), 0.5, 6, "cc.flatten", 10.0)])
 def test_cc_mask_stage_times(m, dims, kind, conn, stage, limit):
     n = dims[0] * dims[1] * dims[2]
     if kind == "checker":
