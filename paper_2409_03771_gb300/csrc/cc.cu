@@ -126,6 +126,33 @@ __device__ __forceinline__ void union_g(int32_t* L, int32_t a, int32_t b, int32_
     record_error(status, MSC_ERR_INTERNAL);
 }
 
+// The same, both ends climbing together until they meet or are both roots:
+// half the round trips where both paths have a few steps, as between the
+// tiles of a noisy mask.
+__device__ __forceinline__ void union_g_together(int32_t* L, int32_t a, int32_t b, int32_t* status) {
+    for (uint32_t it = 0; it < kUnionLimit; ++it) {
+        for (uint32_t hop = 0; hop < kUnionLimit; ++hop) {
+            const int32_t pa = ld_cached_s32(L + a), pb = ld_cached_s32(L + b);
+            if (pa == pb) return;
+            if (pa == a && pb == b) break;
+            const int32_t ga = ld_cached_s32(L + pa), gb = ld_cached_s32(L + pb);
+            if (ga != pa) atomicMin(L + a, ga);
+            if (gb != pb) atomicMin(L + b, gb);
+            a = ga;
+            b = gb;
+        }
+        if (a > b) {
+            const int32_t t = a;
+            a = b;
+            b = t;
+        }
+        const int32_t old = atomicMin(L + b, a);
+        if (old == b) return;
+        b = old;  // below b, fresh from L2
+    }
+    record_error(status, MSC_ERR_INTERNAL);
+}
+
 // Eight mask bytes as eight bits: bit j set iff byte j is nonzero and
 // j < valid.  Rows of any alignment load whole 4-byte words, shifted into
 // place; only words wholly inside the mask are loaded, the few bytes at its
@@ -338,30 +365,36 @@ __global__ void __launch_bounds__(kThreads, MSC_CC_LOCAL_MIN_BLOCKS) k_cc_local(
 // of the grid.
 constexpr int kHaloRows = (CY + 1) * (CZ + 1);  // 81, row y + 9 z
 constexpr int kMergeWarps = 8;
-constexpr uint32_t kMergeQueue = 256;  // contacts of a tile; the rest is united at once
+constexpr uint32_t kMergeQueue = 256;  // contacts of a tile held before they are united
 
 // Unites the tile-local roots of the two ends of a contact: x, y, z of the
 // voxel in the tile and the offset, packed.
+template <bool FEW>
 __device__ __forceinline__ void merge_contact(int32_t* label, const CcGrid& g, int64_t tbase, uint32_t c, int32_t* status) {
     const int64_t nxy = (int64_t)g.nx * g.ny;
     const int64_t v = tbase + (c & 63) + (int64_t)g.nx * (c >> 6 & 7) + nxy * (c >> 9 & 7);
     const int64_t u = v + (c >> 12 & 1) + (int64_t)g.nx * (c >> 13 & 1) + nxy * (c >> 14 & 1);
     const int32_t a = ld_volatile_s32(label + v), b = ld_volatile_s32(label + u);
-    if (a != b) union_g(label, a, b, status);
+    if (a == b) return;
+    if (FEW) union_g_together(label, a, b, status);
+    else union_g(label, a, b, status);
 }
 
-template <bool MASK8>
+// FEW: at most one tile per resident warp, so the round trips of a tile's
+// unions are what the kernel takes (90^3, half of the voxels set at random: 32 ->
+// 28 us with 6 neighbours).  Larger grids read rows of one tile under the
+// unions of others, and the second climb's code costs the reading more than
+// it saves (1024^3, top 10 %: 425 -> 447 us).
+template <bool MASK8, bool FEW>
 __global__ void __launch_bounds__(kMergeWarps * 32, 4) k_cc_merge(const uint8_t* __restrict__ mask, const CcGrid g,
                                                                int32_t* label, int32_t* status) {
     __shared__ uint64_t s_rows[kMergeWarps][kHaloRows];
     __shared__ uint8_t s_next[kMergeWarps][kHaloRows];  // the voxel at x0 + 64
     __shared__ uint16_t s_queue[kMergeWarps][kMergeQueue];
-    __shared__ uint32_t s_count[kMergeWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint64_t* rows = s_rows[warp];
     uint8_t* next = s_next[warp];
     uint16_t* queue = s_queue[warp];
-    uint32_t* count = &s_count[warp];
     const int64_t nxy = (int64_t)g.nx * g.ny;
     const uint32_t first = blockIdx.x * kMergeWarps + warp, step = gridDim.x * kMergeWarps;
     TileWalk tile(g.tx, g.ty, first, step);
@@ -400,7 +433,6 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 4) k_cc_merge(const uint8_t*
                 next[r] = in && __ldg(mask + tbase + CX + (int64_t)g.nx * ly + nxy * lz) != 0;
             }
         }
-        if (lane == 0) *count = 0;
         __syncwarp();
         // +x face crossings as bit y + 8 z, thinned to the first of each patch
         uint64_t xheads;
@@ -411,8 +443,14 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 4) k_cc_merge(const uint8_t*
             const uint64_t X = (uint64_t)xb << 32 | xa;
             xheads = X & ~((X & 0x7f7f7f7f7f7f7f7full) << 1) & ~(X << 8);
         }
-        // each lane's contacts, kind by kind, into the queue
+        // each lane's contacts, kind by kind, into the queue; all lanes unite what it holds
         const int kinds = g.conn == 6 ? 3 : 11;
+        uint32_t total = 0;
+        auto drain = [&](uint32_t count) {
+            __syncwarp();
+            for (uint32_t i = lane; i < count; i += 32) merge_contact<FEW>(label, g, tbase, queue[i], status);
+            __syncwarp();
+        };
 #pragma unroll 1
         for (int kind = 0; kind < kinds; ++kind) {
             uint64_t seg = 0;
@@ -452,17 +490,16 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 4) k_cc_merge(const uint8_t*
                 seg = o & ~(o << 1);
                 c = ly << 6 | lz << 9 | (d == 0 ? 3u : d == 1 ? 5u : d == 2 ? 6u : 7u) << 12;
             }
-            for (; seg; seg &= seg - 1) {
-                const uint32_t code = c | (uint32_t)(__ffsll((long long)seg) - 1);
-                const uint32_t at = atomicAdd(count, 1u);
-                if (at < kMergeQueue) queue[at] = (uint16_t)code;
-                else merge_contact(label, g, tbase, code, status);
+            for (uint32_t act; (act = __ballot_sync(0xffffffffu, seg != 0ull)) != 0u; seg &= seg - 1) {
+                if (total + 32 > kMergeQueue) {  // isolated voxels on both sides of the faces
+                    drain(total);
+                    total = 0;
+                }
+                if (seg) queue[total + __popc(act & lanemask_lt())] = (uint16_t)(c | (uint32_t)(__ffsll((long long)seg) - 1));
+                total += __popc(act);
             }
         }
-        __syncwarp();
-        const uint32_t total = min(*count, kMergeQueue);
-        for (uint32_t i = lane; i < total; i += 32) merge_contact(label, g, tbase, queue[i], status);
-        __syncwarp();
+        drain(total);
     }
 }
 
@@ -779,7 +816,9 @@ int run_cc_mask(const uint8_t* mask, msc_grid gd, int conn, int32_t* label, int3
     const bool mask8 = gd.nx % 8 == 0 && ((uintptr_t)mask & 7) == 0;
     const int sms = current_device().sms;
     auto local = mask8 ? k_cc_local<true> : k_cc_local<false>;
-    auto merge = mask8 ? k_cc_merge<true> : k_cc_merge<false>;
+    const bool few = g.ntiles <= (int64_t)sms * 4 * kMergeWarps;
+    auto merge = mask8 ? (few ? k_cc_merge<true, true> : k_cc_merge<true, false>)
+                       : (few ? k_cc_merge<false, true> : k_cc_merge<false, false>);
     int occ = 1;
     MSC_TRY(max_blocks_per_sm(&occ, local, kThreads, 0));
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)sms * std::max(occ, 1)));

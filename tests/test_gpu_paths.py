@@ -374,9 +374,10 @@ def test_cc_mask_small_grids(m, oracle_mod, conn, dims, density, offset):
 
 
 # (mask, 6 or 14 neighbours, stage, us per call): between what the stage takes and what it took with finds one after
-# the other and run starts from masks (1550 and 2270 us) or in chunks of 8192 voxels (14 us)
+# the other and run starts from masks (1550, 2270 and 104 us) or in chunks of 8192 voxels (14 us)
 @pytest.mark.parametrize("dims,kind,conn,stage,limit", [((512, 512, 512), 0.5, 6, "cc.local", 1300.0),
                                                         ((512, 512, 512), 0.5, 14, "cc.local", 1900.0),
+                                                        ((203, 150, 177), "checker", 14, "cc.merge", 85.0),
                                                         ((48, 48, 48), 0.5, 6, "cc.flatten", 10.0)])
 def test_cc_mask_stage_times(m, dims, kind, conn, stage, limit):
     n = dims[0] * dims[1] * dims[2]
