@@ -32,7 +32,6 @@
 
 #include <algorithm>
 
-#include "coop.cuh"
 #include "msid.cuh"
 #include "radix.cuh"
 
@@ -40,10 +39,10 @@ namespace msc {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr unsigned long long kEmpty = ~0ull;
+constexpr unsigned long long kEmpty = kPairEmpty;
 constexpr uint32_t kSpread = 64;  // random spread of a pair around its home slot (six bits of a hash)
 constexpr uint32_t kCacheResidentSlots = 1u << 20;  // 8 MiB of keys: plain random hashing
-constexpr uint32_t kPad = 4096;   // slots past the capacity: probing never wraps
+constexpr uint32_t kPad = kPairPad;  // slots past the capacity: probing never wraps
 constexpr int kChunkLog2 = 12;    // route (a): chunks of 4096 slots (bases)
 constexpr int kChunk = 1 << kChunkLog2;
 constexpr uint32_t kMaxWindow = 2048;                 // route (a): largest M it accepts
@@ -52,13 +51,12 @@ constexpr int kWinPer = (kChunk + kMaxWindow) / kRankThreads;  // window slots p
 constexpr int kGroupMax = 128;        // route (a): pairs of one base ranked by counting
 
 // control words (ctl[0..3] are shared with the callers: nmin, nmax, cap, K)
-constexpr int kCtlRoute = 16;   // 0: route (a); nonzero: route (b)
+constexpr int kCtlRoute = kPairCtlRoute;   // 0: route (a); nonzero: route (b)
 constexpr int kCtlM = 17;       // largest slot - asc * cap / n of a pair
-constexpr int kCtlCompact = 18; // route (b): compacted pairs
+constexpr int kCtlCompact = kPairCtlCount;  // route (b): compacted pairs
 constexpr int kCtlShift = 19;   // b of the pair keys
 constexpr int kCtlHome = 20;    // home slots of a table too big for the cache: 0 by the minimum, 1 by both labels
 constexpr int kCtlSkip = 21;    // a stage before this one gave up a wait: no pairs are inserted, ms holds no slots
-constexpr int kCtlBarrier = 40; // two grid barriers of the pair sort, zero at its start
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
     // 64-bit finaliser of MurmurHash3
@@ -582,115 +580,6 @@ __global__ void __launch_bounds__(kRankThreads, 2) k_ms_chunk_rank(const unsigne
     }
 }
 
-// Route (b) in one cooperative launch: compact the occupied slots into
-// (key, slot) pairs (each thread scans 8 consecutive slots with 16-byte
-// loads, one atomic append per block and chunk), radix-sort the pairs by key
-// and write table_vals[slot] = rank of the slot's key.  As separate launches
-// the five to seven passes over the few thousand to few million pairs of a
-// usual field took some 20 us each, nearly all of it launch and look-back
-// latency (64^3 field with noise: 93 us as nine launches, 45 as one).  Only as many blocks as there are tiles of
-// pairs take part in the sort; a single tile needs no barrier at all.
-constexpr int kCompactPer = 8;
-constexpr int kPairItems = 8;
-using PairSmem = CoopSmem<unsigned long long, kPairItems>;
-
-struct PairArgs {
-    const unsigned long long* table;
-    uint32_t* ctl;
-    unsigned long long* keys[2];
-    int32_t* slots[2];
-    uint32_t* vals;
-    int npass;
-    int keep_keys;      // the caller reads the sorted keys
-    uint32_t* scratch;  // kCoopScratchWords
-    int32_t* status;
-};
-
-__global__ void __launch_bounds__(kCoopThreads) k_ms_pairs(const PairArgs a) {
-    extern __shared__ __align__(16) uint8_t pair_smem[];
-    PairSmem& S = *reinterpret_cast<PairSmem*>(pair_smem);
-    __shared__ uint32_t s_warp[kCoopWarps];
-    __shared__ uint32_t s_base;
-    if (a.ctl[kCtlRoute] == 0u) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    {
-        const int64_t slots = (int64_t)a.ctl[2] + kPad;
-        constexpr int64_t kChunkSlots = (int64_t)kCoopThreads * kCompactPer;
-        const int64_t nchunks = (slots + kChunkSlots - 1) / kChunkSlots;
-        for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-            const int64_t i0 = c * kChunkSlots + (int64_t)tid * kCompactPer;
-            unsigned long long k[kCompactPer];
-            if (i0 + kCompactPer <= slots) {  // cap and kPad are multiples of 8: whole groups
-#pragma unroll
-                for (int q = 0; q < kCompactPer / 2; ++q) {
-                    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(a.table + i0)[q];
-                    k[2 * q] = v.x;
-                    k[2 * q + 1] = v.y;
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < kCompactPer; ++j) k[j] = i0 + j < slots ? a.table[i0 + j] : kEmpty;
-            }
-            uint32_t cnt = 0;
-#pragma unroll
-            for (int j = 0; j < kCompactPer; ++j) cnt += k[j] != kEmpty;
-            uint32_t incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            if (lane == 31) s_warp[warp] = incl;
-            __syncthreads();
-            if (tid == 0) {
-                uint32_t run = 0;
-                for (int w = 0; w < kCoopWarps; ++w) {
-                    const uint32_t t = s_warp[w];
-                    s_warp[w] = run;
-                    run += t;
-                }
-                s_base = run ? atomicAdd(&a.ctl[kCtlCompact], run) : 0u;
-            }
-            __syncthreads();
-            uint32_t pos = s_base + s_warp[warp] + incl - cnt;
-#pragma unroll
-            for (int j = 0; j < kCompactPer; ++j) {
-                if (k[j] != kEmpty) {
-                    MSC_GUARD(pos < (uint32_t)slots, a.status, -131) {
-                        a.keys[0][pos] = k[j];
-                        a.slots[0][pos] = (int32_t)(i0 + j);
-                    }
-                    ++pos;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    GridBarrier all{a.ctl + kCtlBarrier, gridDim.x, 0};
-    if (!grid_barrier(all, a.status)) return;
-    const uint32_t K = __ldcg(a.ctl + kCtlCompact);
-    const uint32_t active = min(gridDim.x, (K + PairSmem::kTile - 1) / PairSmem::kTile);
-    if (blockIdx.x >= active) return;
-    GridBarrier bar{a.ctl + kCtlBarrier + 1, active, 0};
-#pragma unroll 1
-    for (int p = 0; p < a.npass; ++p) {
-        const bool last = p + 1 == a.npass;
-        const unsigned long long* kin = a.keys[p & 1];
-        const int32_t* vin = a.slots[p & 1];
-        unsigned long long* kout = a.keys[(p & 1) ^ 1];
-        int32_t* vout = a.slots[(p & 1) ^ 1];
-        const CoopPass r = coop_radix_pass<unsigned long long, kPairItems>(
-            S, K, 8 * p, false, [&](uint32_t i) { return kin[i]; }, [&](uint32_t i) { return (uint32_t)vin[i]; },
-            [&](uint32_t pos, unsigned long long k, uint32_t slot) {
-                if (!last || a.keep_keys) kout[pos] = k;
-                if (!last) vout[pos] = (int32_t)slot;
-                else a.vals[slot] = pos;
-            },
-            a.scratch, bar, a.status);
-        if (r == kPassFailed) return;
-    }
-}
-
 // ms[v] = vals[ms[v]]: 8 vertices per thread, lane-consecutive, so the
 // gathers of a warp fall on neighbouring slots.
 constexpr int kLookupPer = 8;
@@ -829,34 +718,20 @@ int run_ms_id(const int32_t* asc, const int32_t* desc, int32_t n, int32_t* ms, i
     }
     // route (b), run when the flag asks for it (returns at once otherwise)
     {
-        PairArgs a{};
-        a.table = sc.table_keys;
-        a.ctl = sc.ctl;
+        PairRanks p{};
+        p.table = sc.table_keys;
+        p.ctl = sc.ctl;
         for (int i = 0; i < 2; ++i) {
-            a.keys[i] = sc.ukeys[i];
-            a.slots[i] = sc.uvals[i];
+            p.keys[i] = sc.ukeys[i];
+            p.slots[i] = sc.uvals[i];
         }
-        a.vals = sc.table_vals;
-        a.npass = std::max(1, (2 * sh + 7) / 8);
-        a.keep_keys = ranked ? 1 : 0;
-        a.scratch = sc.sort.ord_cnt;
-        a.status = status;
-        static int configured_dev = -1;
-        if (configured_dev != current_device().id) {
-            MSC_TRY(cudaFuncSetAttribute(k_ms_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PairSmem)));
-            configured_dev = current_device().id;
-        }
-        int blocks = 0;
-        const int r = coop_blocks(k_ms_pairs, kCoopThreads, sizeof(PairSmem),
-                                  std::min<int64_t>(ceil_div(n, PairSmem::kTile), kCoopMaxBlocks), &blocks);
+        p.vals = sc.table_vals;
+        p.npass = std::max(1, (2 * sh + 7) / 8);
+        p.keep_keys = ranked ? 1 : 0;
+        const int r = run_pair_ranks(p, n, sc.sort, status, s);
         if (r) return r;
-        {
-            TraceScope ts_("msid.pairs", s);
-            const int rr = coop_launch(k_ms_pairs, blocks, kCoopThreads, sizeof(PairSmem), s, a);
-            if (rr) return rr;
-        }
         if (ranked) {
-            *ranked = MsRanked{sc.ukeys[a.npass & 1], sc.table_vals, sc.ctl + kCtlSkip};
+            *ranked = MsRanked{sc.ukeys[p.npass & 1], sc.table_vals, sc.ctl + kCtlSkip};
             return MSC_OK;
         }
     }

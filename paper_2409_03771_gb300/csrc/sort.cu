@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <utility>
 
+#include "coop.cuh"
 #include "radix.cuh"
 #include "sort.cuh"
 #include "tma.cuh"
@@ -56,21 +57,21 @@ constexpr int kCounterWords = 8 + kMaxBuckets * kFillStride;  // tile counters, 
 // sixteen consecutive keys per thread (128-byte lane stride), 0.16 now.
 constexpr int kHistPairs = 8;  // 16-byte loads in flight per thread
 
-__global__ void __launch_bounds__(256) k_hist(const unsigned long long* __restrict__ keys, int64_t n_host,
-                                              const int32_t* __restrict__ d_n, int npass, uint32_t* __restrict__ hist) {
-    extern __shared__ uint32_t sh[];  // [kWarps][npass][256]
+// sh: [kWarps][npass][256].  (Loads past the L1: in the pair ranks' kernel the
+// keys were written by other blocks.)
+__device__ __forceinline__ void add_digit_counts(const unsigned long long* keys, int64_t n, int npass, uint32_t* hist,
+                                                 uint32_t* sh) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < kWarps * npass * kBins; i += blockDim.x) sh[i] = 0;
     __syncthreads();
     uint32_t* wsh = sh + warp * npass * kBins;
-    const int64_t n = d_n ? min((int64_t)*d_n, n_host) : n_host;
     constexpr int64_t kStep = 2 * 256 * kHistPairs;
     for (int64_t b = (int64_t)blockIdx.x * kStep; b < n; b += (int64_t)gridDim.x * kStep) {
         if (b + kStep <= n) {
             ulonglong2 k[kHistPairs];
 #pragma unroll
             for (int q = 0; q < kHistPairs; ++q)
-                k[q] = __ldg(reinterpret_cast<const ulonglong2*>(keys + b) + q * 256 + tid);
+                k[q] = __ldcg(reinterpret_cast<const ulonglong2*>(keys + b) + q * 256 + tid);
             for (int p = 0; p < npass; ++p) {
                 uint32_t* h = wsh + p * kBins;
 #pragma unroll
@@ -94,6 +95,12 @@ __global__ void __launch_bounds__(256) k_hist(const unsigned long long* __restri
         for (int w = 0; w < kWarps; ++w) c += sh[w * npass * kBins + i];
         if (c) atomicAdd(&hist[i], c);
     }
+}
+
+__global__ void __launch_bounds__(256) k_hist(const unsigned long long* __restrict__ keys, int64_t n_host,
+                                              const int32_t* __restrict__ d_n, int npass, uint32_t* __restrict__ hist) {
+    extern __shared__ uint32_t sh[];
+    add_digit_counts(keys, d_n ? min((int64_t)*d_n, n_host) : n_host, npass, hist, sh);
 }
 
 // Per-segment histograms of the float keys for the 4 passes of a
@@ -182,6 +189,7 @@ struct PassArgs {
     const int32_t* seg_tile0;
     int64_t seg_tiles;
     int seg_stride;
+    uint32_t* rank_of;  // RANK pass: rank_of[payload] = position; keys_out may be null
 };
 
 // Keys per thread: 64-bit sorts take 24 at two blocks per SM (six passes over
@@ -209,13 +217,13 @@ constexpr size_t pass_smem_bytes() {
 // the segment's first tile, bin starts come per segment, and positions are
 // segment-local (keys land at seg_off + position; order gets the position).
 //
-// VALS: with a payload; without, keys alone are moved.
-template <typename KeyT, bool FROM_F, bool BUCKET, bool SEG, bool VALS>
-__global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_onesweep(const PassArgs<KeyT> a) {
+// VALS: with a payload; without, keys alone are moved.  RANK: the payload's
+// position goes to rank_of instead.
+template <typename KeyT, bool FROM_F, bool BUCKET, bool SEG, bool VALS, bool RANK>
+__device__ __forceinline__ void onesweep_tiles(const PassArgs<KeyT>& a, uint8_t* smem) {
     constexpr int kItems = kPassItems<KeyT>, kTile = kThreads * kItems;
     static_assert(kTile >= kSortTile, "the look-back words are sized for tiles of kSortTile keys");
     static_assert(!SEG || kTile == kSortTile, "a segment's tiles and histograms are those of its table");
-    extern __shared__ __align__(16) uint8_t smem[];
     uint32_t* s_whist = reinterpret_cast<uint32_t*>(smem);  // [kWarps][256]
     uint32_t* s_match = s_whist + kWarps * kBins;          // [kWarps][256] lanes per digit, 0 between keys
     uint32_t* s_total = s_match + kWarps * kBins;          // [256]
@@ -420,20 +428,31 @@ __global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_oneswee
                 }
             } else {
                 KeyT* kout = a.keys_out + seg_base;
-                int32_t* vout = VALS ? a.vals_out + seg_base : nullptr;
+                int32_t* vout = VALS && !RANK ? a.vals_out + seg_base : nullptr;
                 for (int i = tid; i < cnt; i += kThreads) {
                     const KeyT kk = s_keys[i];
                     const uint32_t d = (uint32_t)(kk >> a.shift) & 255u;
                     const uint32_t pos = s_gbase[d] + (uint32_t)i - s_excl[d];
                     MSC_GUARD(pos < (uint64_t)n, a.status, -102) {
-                        kout[pos] = kk;
-                        if constexpr (VALS) vout[pos] = s_vals[i];
+                        if constexpr (RANK) {
+                            if (a.keys_out) kout[pos] = kk;
+                            a.rank_of[s_vals[i]] = pos;
+                        } else {
+                            kout[pos] = kk;
+                            if constexpr (VALS) vout[pos] = s_vals[i];
+                        }
                     }
                 }
             }
         }
         __syncthreads();
     }
+}
+
+template <typename KeyT, bool FROM_F, bool BUCKET, bool SEG, bool VALS>
+__global__ void __launch_bounds__(kThreads, sizeof(KeyT) == 8 ? 2 : 3) k_onesweep(const PassArgs<KeyT> a) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    onesweep_tiles<KeyT, FROM_F, BUCKET, SEG, VALS, false>(a, smem);
 }
 
 // Width of the id buckets the last pass files pairs into: 2^19 ids at
@@ -476,6 +495,167 @@ int launch_pass(const PassArgs<KeyT>& a, int64_t max_n, cudaStream_t s, const ch
     }
     MSC_LAUNCHED();
     return MSC_OK;
+}
+
+// Ranks of a hash table's keys in one cooperative launch: compact the occupied
+// slots into (key, slot) pairs (each thread scans 8 consecutive slots with
+// 16-byte loads, one atomic append per block and chunk), radix-sort the pairs
+// by key and write vals[slot] = rank of the slot's key.  As separate launches
+// the five to seven passes over the few thousand to few million pairs of a
+// usual field took some 20 us each, nearly all of it launch and look-back
+// latency (64^3 field with noise: 93 us as nine launches, 45 as one).
+//
+// Up to kPairsCoopMax pairs the digit passes are those of coop.cuh, by only as
+// many of the at most two blocks per SM as there are tiles of pairs; a single
+// tile needs no barrier at all.  More pairs go through onesweep passes in the
+// same launch, whose tiles are read once per pass and three times as large.
+// us with the passes of coop.cuh / onesweep passes (the launches of before):
+//   490 000 pairs 88 / 122, 810 000 146 / 137, 1.2M 160 / 157, 2.6M 305 / 258,
+//   9.1M 834 / 677, 23.4M 2921 / 2121 (2010), 46.5M 5685 / 4030 (3670).
+// Per pass the first read and write 32 bytes per pair (24 with one tile per
+// block), the others 24.
+constexpr int kCompactPer = 8;
+constexpr int kPairItems = 8;
+using PairSmem = CoopSmem<unsigned long long, kPairItems>;
+constexpr int kPairTile = kThreads * kPassItems<unsigned long long>;
+constexpr uint32_t kPairsCoopMax = 1u << 20;
+// The kernel that holds both ways takes 96 KB of shared memory per block, and 5 us
+// more where there are few pairs (43 against 49 for 3600): up to this many
+// vertices, where a field has at most kPairsCoopMax pairs (white noise: a
+// third of its vertices), the one with the passes of coop.cuh alone.
+constexpr int64_t kPairsCoopVertices = 3 << 20;
+static_assert(kCoopThreads == kThreads, "one block shape for both sorts");
+
+struct PairArgs {
+    PairRanks p;
+    uint32_t* scratch;             // kCoopScratchWords
+    uint32_t* hist;                // [npass][256] ONESWEEP
+    uint32_t* tile_counters;       // [npass] ONESWEEP
+    unsigned long long* lookback;  // ONESWEEP
+    int32_t* status;
+};
+
+template <bool ONESWEEP>
+__global__ void __launch_bounds__(kCoopThreads, 2) k_pair_ranks(const PairArgs args) {
+    extern __shared__ __align__(16) uint8_t pair_smem[];
+    PairSmem& S = *reinterpret_cast<PairSmem*>(pair_smem);
+    const PairRanks& a = args.p;
+    int32_t* status = args.status;
+    __shared__ uint32_t s_warp[kCoopWarps];
+    __shared__ uint32_t s_base;
+    if (a.ctl[kPairCtlRoute] == 0u) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    {
+        const int64_t slots = (int64_t)a.ctl[2] + kPairPad;
+        constexpr int64_t kChunkSlots = (int64_t)kCoopThreads * kCompactPer;
+        const int64_t nchunks = (slots + kChunkSlots - 1) / kChunkSlots;
+        for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
+            const int64_t i0 = c * kChunkSlots + (int64_t)tid * kCompactPer;
+            unsigned long long k[kCompactPer];
+            if (i0 + kCompactPer <= slots) {  // capacity and pad are multiples of 8: whole groups
+#pragma unroll
+                for (int q = 0; q < kCompactPer / 2; ++q) {
+                    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(a.table + i0)[q];
+                    k[2 * q] = v.x;
+                    k[2 * q + 1] = v.y;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kCompactPer; ++j) k[j] = i0 + j < slots ? a.table[i0 + j] : kPairEmpty;
+            }
+            uint32_t cnt = 0;
+#pragma unroll
+            for (int j = 0; j < kCompactPer; ++j) cnt += k[j] != kPairEmpty;
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane == 31) s_warp[warp] = incl;
+            __syncthreads();
+            if (tid == 0) {
+                uint32_t run = 0;
+                for (int w = 0; w < kCoopWarps; ++w) {
+                    const uint32_t t = s_warp[w];
+                    s_warp[w] = run;
+                    run += t;
+                }
+                s_base = run ? atomicAdd(&a.ctl[kPairCtlCount], run) : 0u;
+            }
+            __syncthreads();
+            uint32_t pos = s_base + s_warp[warp] + incl - cnt;
+#pragma unroll
+            for (int j = 0; j < kCompactPer; ++j) {
+                if (k[j] != kPairEmpty) {
+                    MSC_GUARD(pos < (uint32_t)slots, status, -131) {
+                        a.keys[0][pos] = k[j];
+                        a.slots[0][pos] = (int32_t)(i0 + j);
+                    }
+                    ++pos;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    GridBarrier all{a.ctl + kPairCtlBarrier, gridDim.x, 0};
+    if (!grid_barrier(all, status)) return;
+    const uint32_t K = __ldcg(a.ctl + kPairCtlCount);
+    if (ONESWEEP && K > kPairsCoopMax) {
+        const int64_t words = ((int64_t)K + kPairTile - 1) / kPairTile * kBins;
+        for (int64_t i = (int64_t)blockIdx.x * kCoopThreads + tid; i < words; i += (int64_t)gridDim.x * kCoopThreads)
+            args.lookback[i] = 0;
+        for (int i = blockIdx.x * kCoopThreads + tid; i < a.npass * kBins; i += gridDim.x * kCoopThreads) args.hist[i] = 0;
+        if (blockIdx.x == 0 && tid < a.npass) args.tile_counters[tid] = 0;
+        if (!grid_barrier(all, status)) return;
+        add_digit_counts(a.keys[0], K, a.npass, args.hist, reinterpret_cast<uint32_t*>(pair_smem));
+        if (!grid_barrier(all, status)) return;
+        PassArgs<unsigned long long> w{};
+        w.n = K;
+        w.lookback = args.lookback;
+        w.status = status;
+        w.rank_of = a.vals;
+#pragma unroll 1
+        for (int p = 0; p < a.npass; ++p) {
+            const int in = p & 1;
+            w.keys_in = in ? a.keys[1] : a.keys[0];
+            w.vals_in = in ? a.slots[1] : a.slots[0];
+            w.keys_out = in ? a.keys[0] : a.keys[1];
+            w.vals_out = in ? a.slots[0] : a.slots[1];
+            w.hist = args.hist + p * kBins;
+            w.shift = 8 * p;
+            w.tile_counter = args.tile_counters + p;
+            w.epoch = (uint32_t)(p + 1);
+            if (p + 1 < a.npass) {
+                onesweep_tiles<unsigned long long, false, false, false, true, false>(w, pair_smem);
+                if (!grid_barrier(all, status)) return;
+            } else {
+                if (!a.keep_keys) w.keys_out = nullptr;
+                onesweep_tiles<unsigned long long, false, false, false, true, true>(w, pair_smem);
+            }
+        }
+        return;
+    }
+    const uint32_t active = min(gridDim.x, (K + PairSmem::kTile - 1) / PairSmem::kTile);
+    if (blockIdx.x >= active) return;
+    GridBarrier bar{a.ctl + kPairCtlBarrier + 1, active, 0};
+#pragma unroll 1
+    for (int p = 0; p < a.npass; ++p) {
+        const bool last = p + 1 == a.npass;
+        const unsigned long long* kin = a.keys[p & 1];
+        const int32_t* vin = a.slots[p & 1];
+        unsigned long long* kout = a.keys[(p & 1) ^ 1];
+        int32_t* vout = a.slots[(p & 1) ^ 1];
+        const CoopPass r = coop_radix_pass<unsigned long long, kPairItems>(
+            S, K, 8 * p, false, [&](uint32_t i) { return kin[i]; }, [&](uint32_t i) { return (uint32_t)vin[i]; },
+            [&](uint32_t pos, unsigned long long k, uint32_t slot) {
+                if (!last || a.keep_keys) kout[pos] = k;
+                if (!last) vout[pos] = (int32_t)slot;
+                else a.vals[slot] = pos;
+            },
+            args.scratch, bar, status);
+        if (r == kPassFailed) return;
+    }
 }
 
 }  // namespace
@@ -658,6 +838,28 @@ int run_sort_u64(unsigned long long* keys, int32_t* vals, unsigned long long* ke
     }
     *result_in_alt = (npass & 1) != 0;
     return MSC_OK;
+}
+
+template <bool ONESWEEP>
+static int launch_pair_ranks(const PairArgs& a, int64_t n, cudaStream_t s) {
+    constexpr size_t smem = ONESWEEP ? std::max(sizeof(PairSmem), pass_smem_bytes<unsigned long long, true>()) : sizeof(PairSmem);
+    static_assert(!ONESWEEP || smem >= (size_t)kWarps * 8 * kBins * sizeof(uint32_t), "the digit counts fit too");
+    auto kern = k_pair_ranks<ONESWEEP>;
+    static int configured_dev = -1;
+    if (configured_dev != current_device().id) {
+        MSC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        configured_dev = current_device().id;
+    }
+    int blocks = 0;
+    const int r = coop_blocks(kern, kCoopThreads, smem, std::min<int64_t>(ceil_div(n, PairSmem::kTile), kCoopMaxBlocks), &blocks);
+    if (r) return r;
+    TraceScope ts_("msid.pairs", s);
+    return coop_launch(kern, blocks, kCoopThreads, smem, s, a);
+}
+
+int run_pair_ranks(const PairRanks& p, int64_t n, const SortScratch& sc, int32_t* status, cudaStream_t s) {
+    const PairArgs a{p, sc.ord_cnt, sc.hist, sc.tile_counters, sc.lookback, status};
+    return n > kPairsCoopVertices ? launch_pair_ranks<true>(a, n, s) : launch_pair_ranks<false>(a, n, s);
 }
 
 }  // namespace msc

@@ -59,6 +59,28 @@ int run_order_seg(const float* f, const SegTable& t, int32_t* order, uint32_t* k
                   uint32_t* key_b, int32_t* id_b, const SortScratch& sc, int32_t* status,
                   cudaStream_t s);
 
+// The occupied slots of a hash table of 64-bit keys (kPairEmpty: free), ranked:
+// vals[slot] = rank of the slot's key, and keys[npass & 1] the sorted keys with
+// keep_keys.  On the device, ctl holds the table's capacity [2] (slots:
+// capacity + kPairPad), whether there is anything to do [kPairCtlRoute] and
+// two barrier words that are 0 [kPairCtlBarrier]; ctl[kPairCtlCount], 0 at the
+// start, gets the number of keys.  At most n keys; buffers of n + kPairPad.
+constexpr unsigned long long kPairEmpty = ~0ull;
+constexpr uint32_t kPairPad = 4096;
+constexpr int kPairCtlRoute = 16, kPairCtlCount = 18, kPairCtlBarrier = 40;
+
+struct PairRanks {
+    const unsigned long long* table;
+    uint32_t* ctl;
+    unsigned long long* keys[2];
+    int32_t* slots[2];
+    uint32_t* vals;
+    int npass;      // 8-bit digits of the keys
+    int keep_keys;  // the caller reads the sorted keys
+};
+
+int run_pair_ranks(const PairRanks& p, int64_t n, const SortScratch& sc, int32_t* status, cudaStream_t s);
+
 // Stable sort of (keys, vals) by the low `key_bits` bits of keys.  The
 // count is read on the device from *d_count (<= max_count).  Returns, via
 // *result_in_alt, whether the sorted data ended in the alt buffers.  With
@@ -66,6 +88,6 @@ int run_order_seg(const float* f, const SegTable& t, int32_t* order, uint32_t* k
 int run_sort_u64(unsigned long long* keys, int32_t* vals, unsigned long long* keys_alt,
                  int32_t* vals_alt, const int32_t* d_count, int64_t max_count, int key_bits,
                  const SortScratch& sc, int32_t* status, cudaStream_t s, bool* result_in_alt,
-                 const char* hist_label = "msid.sort_hist", const char* pass_label = "msid.sort_pass");
+                 const char* hist_label, const char* pass_label);
 
 }  // namespace msc

@@ -396,3 +396,72 @@ def test_cc_mask_stage_times(m, dims, kind, conn, stage, limit):
         times.append(m.msc_trace_collect()[stage][1] * 1e3)
     m.msc_trace_reset()
     assert min(times) < limit, times
+
+
+# ---------------------------------------------------------------------------
+# cell ids: pairs on both sides of the count from which on they are sorted by
+# onesweep passes (2^20), with and without the sorted keys
+
+
+def dense_pairs(k, n, gen):
+    """Labels with exactly k distinct pairs: vertex v < k has the pair (v // 1024, 1024-grid column), the rest repeat it."""
+    cols = 1024
+    rows = (k + cols - 1) // cols
+    v = torch.arange(n, device="cuda") % k
+    a, d = v // cols, v % cols
+    # minima sit at [0, rows), maxima at [rows, rows + cols): both label themselves, in pairs of their own
+    asc, desc = a, rows + d
+    return asc.int(), desc.int(), rows, cols
+
+
+@pytest.mark.parametrize("k", [(1 << 20) - 1, 1 << 20, (1 << 20) + 1, (1 << 20) + 6144, 3000000])
+def test_pair_ranks_either_side_of_the_limit(m, k):
+    n = (1 << 22) + 5
+    gen = torch.Generator(device="cuda").manual_seed(k)
+    ids = torch.randperm(n, device="cuda", generator=gen)
+    asc, desc, rows, cols = dense_pairs(k, n, gen)
+    # shuffled vertices, roots included: every label's own vertex keeps it
+    amap, dmap = ids[:rows], ids[rows:rows + cols]
+    lab = [amap[asc.long()], dmap[(desc - rows).long()]]
+    for x, r in zip(lab, (amap, dmap)):
+        x[r] = r
+    keys, want = torch.unique(lab[0] * n + lab[1], return_inverse=True)
+    assert abs(keys.numel() - k) <= 2 * (rows + cols)
+    ms, got = m.ms_id(lab[0].int(), lab[1].int())
+    assert got == keys.numel()
+    assert torch.equal(ms.long(), want)
+
+
+@pytest.mark.parametrize("dims", [[(150, 140, 130)], [(64, 64, 64), (201, 190, 77), (5, 3, 2), (128, 128, 127)],
+                                  [(100, 99, 98)] * 5])
+def test_batch_of_noise_with_many_pairs(m, dims):
+    """More than 2^20 pairs in one batch or just below: instance by instance as single segmentations."""
+    b = m.Batch(dims)
+    gen = torch.Generator(device="cuda").manual_seed(len(dims))
+    b.f.copy_(torch.rand(b.total, device="cuda", generator=gen))
+    b.plan()
+    for _ in range(2):
+        b.launch()
+    cells = b.num_cells.tolist()
+    for i, d in enumerate(dims):
+        lo, hi = b.offsets[i], b.offsets[i + 1]
+        order, asc, desc, ms, k = m.segment(b.f[lo:hi].clone(), d)
+        assert cells[i] == k
+        for got, want in ((b.order, order), (b.asc, asc), (b.desc, desc), (b.ms, ms)):
+            assert torch.equal(got[lo:hi], want)
+
+
+def test_pair_ranks_time_per_pair(m):
+    """Tens of millions of pairs: 0.09 us per thousand with onesweep passes (0.086 as launches), 0.125 without."""
+    b = m.Batch([(400, 400, 400)])
+    b.f.copy_(torch.rand(b.total, device="cuda", generator=torch.Generator(device="cuda").manual_seed(3)))
+    b.run()
+    times = []
+    for _ in range(4):
+        m.msc_trace_reset()
+        m.msc_trace_enable(True)
+        b.run()
+        m.msc_trace_enable(False)
+        times.append(m.msc_trace_collect()["msid.pairs"][1] * 1e6)
+    m.msc_trace_reset()
+    assert min(times) / int(b.num_cells[0]) < 0.108, (times, int(b.num_cells[0]))
