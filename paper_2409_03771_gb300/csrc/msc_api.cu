@@ -4,15 +4,14 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <map>
 #include <mutex>
-#include <tuple>
 
 #include "adjacency.cuh"
 #include "cc.cuh"
 #include "common.cuh"
 #include "compress.cuh"
 #include "msid.cuh"
+#include "remembered.h"
 #include "sort.cuh"
 #include "steepest.cuh"
 #include "tma.cuh"
@@ -41,23 +40,10 @@ const Device& current_device() {
 }
 
 cudaError_t max_blocks_per_sm(int* out, const void* kernel, int threads, size_t smem) {
-    static std::mutex mu;
-    static std::map<std::tuple<int, const void*, int, size_t>, int> known;  // one entry per kernel and launch shape
-    const auto key = std::make_tuple(current_device().id, kernel, threads, smem);
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        const auto it = known.find(key);
-        if (it != known.end()) {
-            *out = it->second;
-            return cudaSuccess;
-        }
-    }
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, threads, smem);
-    if (e == cudaSuccess) {
-        std::lock_guard<std::mutex> lock(mu);
-        known[key] = *out;
-    }
-    return e;
+    static Remembered known;
+    return (cudaError_t)known.get(out, current_device().id, kernel, threads, smem, [&](int* blocks) {
+        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, threads, smem);
+    });
 }
 
 bool make_tensor_map_3d(CUtensorMap* map, const void* base, int elem_bytes, int nx, int ny, int nz,
