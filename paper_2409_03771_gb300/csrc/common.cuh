@@ -146,6 +146,10 @@ cudaError_t max_blocks_per_sm(int* out, K* kernel, int threads, size_t smem) {
     return max_blocks_per_sm(out, reinterpret_cast<const void*>(kernel), threads, smem);
 }
 
+// SMs that kernels on a stream can use: those of the device, or of the
+// stream's green context (a part of the SMs that a program has set aside).
+int stream_sms(cudaStream_t s);
+
 // Bump-pointer carving of a caller workspace (256-byte aligned pieces).
 struct Carver {
     char* base;

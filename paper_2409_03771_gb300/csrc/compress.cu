@@ -353,7 +353,7 @@ int run_compress(int32_t* const* ptrs, int count, int32_t n, const CompressScrat
     auto tail = tune.trusted ? k_jump_tail<false> : k_jump_tail<true>;
     int blocks = 0;
     const int r = coop_blocks(
-        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * tail_blocks_per_sm(n)), &blocks);
+        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * tail_blocks_per_sm(n)), s, &blocks);
     if (r) return r;
     TraceScope ts_("compress.tail", s);
     return coop_launch(tail, blocks, kThreads, 0, s, pr, count, full, steps, build_max, &sc.ctl[0].barrier, status);

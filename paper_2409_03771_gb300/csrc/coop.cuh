@@ -249,18 +249,21 @@ __device__ __forceinline__ CoopPass coop_radix_pass(CoopSmem<KeyT, ITEMS>& S, ui
 // ----------------------------------------------------------------------------
 // host side
 
-// Blocks of a cooperative launch: at most `want`, all resident at once.
+// Blocks of a cooperative launch on a stream: at most `want`, all resident at
+// once on the SMs that the stream has.
 template <typename K>
-int coop_blocks(K kernel, int threads, size_t smem, int64_t want, int* out) {
+int coop_blocks(K kernel, int threads, size_t smem, int64_t want, cudaStream_t s, int* out) {
     int occ = 0;
     MSC_TRY(max_blocks_per_sm(&occ, kernel, threads, smem));
     if (occ < 1) return MSC_ERR_CUDA;
-    *out = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)current_device().sms * occ));
+    *out = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)stream_sms(s) * occ));
     return MSC_OK;
 }
 
-// The kernels here run on any number of blocks: a grid that does not fit (a
-// context confined to a part of the SMs) is halved until it does.
+// The kernels here run on any number of blocks: a grid that the runtime finds
+// too large all the same is halved until it fits.  (While a stream is being
+// captured the launch is not where the size is judged: coop_blocks has to be
+// right.)
 template <typename... P, typename... A>
 int coop_launch(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t s, const A&... args) {
     cudaLaunchConfig_t cfg{};

@@ -46,6 +46,33 @@ cudaError_t max_blocks_per_sm(int* out, const void* kernel, int threads, size_t 
     });
 }
 
+int stream_sms(cudaStream_t s) {
+    using GetCtxFn = CUresult (*)(CUstream, CUgreenCtx*);
+    using GetResourceFn = CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+    static GetCtxFn get_ctx = nullptr;
+    static GetResourceFn get_resource = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &fn, 12040, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            return;
+        void* fn2 = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &fn2, 12040, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            return;
+        get_resource = reinterpret_cast<GetResourceFn>(fn2);
+        get_ctx = reinterpret_cast<GetCtxFn>(fn);
+    });
+    const int sms = current_device().sms;
+    CUgreenCtx ctx = nullptr;
+    CUdevResource res{};
+    if (!get_ctx || get_ctx(reinterpret_cast<CUstream>(s), &ctx) != CUDA_SUCCESS || !ctx) return sms;
+    if (get_resource(ctx, &res, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS || res.sm.smCount == 0) return sms;
+    return std::min(sms, (int)res.sm.smCount);
+}
+
 bool make_tensor_map_3d(CUtensorMap* map, const void* base, int elem_bytes, int nx, int ny, int nz,
                         int bx, int by, int bz) {
     using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,

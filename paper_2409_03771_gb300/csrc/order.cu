@@ -698,7 +698,7 @@ int launch_coop(const CoopOrderArgs& a, cudaStream_t s) {
     }
     int blocks = 0;
     const int r = coop_blocks(k_ord_coop<ITEMS>, kCoopThreads, sizeof(Smem),
-                              std::min<int64_t>(ceil_div(a.n, Smem::kTile), kCoopMaxBlocks), &blocks);
+                              std::min<int64_t>(ceil_div(a.n, Smem::kTile), kCoopMaxBlocks), s, &blocks);
     if (r) return r;
     TraceScope ts_("order.coop", s);
     return coop_launch(k_ord_coop<ITEMS>, blocks, kCoopThreads, sizeof(Smem), s, a);

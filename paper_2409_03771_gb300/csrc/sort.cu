@@ -851,7 +851,8 @@ static int launch_pair_ranks(const PairArgs& a, int64_t n, cudaStream_t s) {
         configured_dev = current_device().id;
     }
     int blocks = 0;
-    const int r = coop_blocks(kern, kCoopThreads, smem, std::min<int64_t>(ceil_div(n, PairSmem::kTile), kCoopMaxBlocks), &blocks);
+    const int r = coop_blocks(kern, kCoopThreads, smem, std::min<int64_t>(ceil_div(n, PairSmem::kTile), kCoopMaxBlocks), s,
+                              &blocks);
     if (r) return r;
     TraceScope ts_("msid.pairs", s);
     return coop_launch(kern, blocks, kCoopThreads, smem, s, a);
