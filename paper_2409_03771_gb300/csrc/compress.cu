@@ -283,14 +283,18 @@ __global__ void __launch_bounds__(kThreads) k_jump_tail(const JumpPair pr, int c
 // 256 x 250 noise: 159 us as thirteen launches, 122 now), but on paths of more
 // than 625 steps the tail goes on with whole sweeps.
 // The tail's grid: two blocks per SM up to 2^21 vertices (a random chain of
-// 10^6: 128 us, 157 with four) and where it has nothing left to do, which
-// leaves room to start beside other streams' kernels; four between, where
-// long paths need them (one path of 10^7 vertices: 476 us with two, 408 with
-// four, 404 as a launch per sweep; 2^24 - 1: 738, 628, 625).
+// 10^6: 128 us, 157 with four), on the pointers of fields and where it has
+// nothing left to do, which leaves room to start beside other streams' kernels
+// (a burst of twelve requests at a server: 2125 us, 2159 with four); four
+// for a caller's own pointers between, where long paths need them (one path
+// of 10^7 vertices: 476 us with two, 408 with four, 404 as a launch per sweep;
+// 2^24 - 1: 738, 628, 625).
 constexpr int64_t kTailVertices = 1 << 20;
 constexpr int64_t kLargeVertices = 1 << 24;
 int full_sweeps(int64_t n) { return n <= kTailVertices ? 0 : n < kLargeVertices ? 4 : 8; }
-int tail_blocks_per_sm(int64_t n) { return n <= 2 * kTailVertices || n >= kLargeVertices ? 2 : 4; }
+int tail_blocks_per_sm(int64_t n, bool trusted) {
+    return trusted || n <= 2 * kTailVertices || n >= kLargeVertices ? 2 : 4;
+}
 
 }  // namespace
 
@@ -353,7 +357,7 @@ int run_compress(int32_t* const* ptrs, int count, int32_t n, const CompressScrat
     auto tail = tune.trusted ? k_jump_tail<false> : k_jump_tail<true>;
     int blocks = 0;
     const int r = coop_blocks(
-        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * tail_blocks_per_sm(n)), s, &blocks);
+        tail, kThreads, 0, std::min<int64_t>(chunks, (int64_t)current_device().sms * tail_blocks_per_sm(n, tune.trusted)), s, &blocks);
     if (r) return r;
     TraceScope ts_("compress.tail", s);
     return coop_launch(tail, blocks, kThreads, 0, s, pr, count, full, steps, build_max, &sc.ctl[0].barrier, status);
