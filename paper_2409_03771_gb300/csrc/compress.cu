@@ -107,7 +107,7 @@ __device__ __forceinline__ uint32_t jump_group(const int32_t* p, int32_t n, cons
 #pragma unroll
     for (int j = 0; j < kPerThread; ++j) {
         if (!(valid >> j & 1u) || d[j] < 0) continue;
-        if (CHECKED && (uint32_t)d[j] >= (uint32_t)n) {
+        if ((uint32_t)d[j] >= (uint32_t)n) {
             record_error(status, MSC_ERR_ARG);
             continue;
         }
@@ -125,10 +125,10 @@ __device__ __forceinline__ uint32_t jump_group(const int32_t* p, int32_t n, cons
             const int32_t u = d[j];
             if (w[j] == u) {
                 live &= ~(1u << j);  // u is a root: done
-            } else if (CHECKED && (uint32_t)w[j] >= (uint32_t)n) {
+            } else if ((uint32_t)w[j] >= (uint32_t)n) {
                 record_error(status, MSC_ERR_ARG);  // out of range or inactive target
                 live &= ~(1u << j);
-            } else if (CHECKED && w[j] == vid[j]) {
+            } else if (w[j] == vid[j]) {
                 record_error(status, MSC_ERR_NOT_CONVERGED);
                 live &= ~(1u << j);
             } else {

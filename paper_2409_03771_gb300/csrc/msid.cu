@@ -4,11 +4,11 @@
 // lexicographic order, minimum first.
 //
 // 1. A linear-probing hash table de-duplicates the pair keys
-//    (asc << b) | desc, b = ceil(log2 n).  Its capacity is a power of two
-//    >= 2 * #minima * #maxima, or >= n when that is more than n (there are
-//    at most n distinct pairs), chosen on the device, so smooth fields (few
-//    extrema) use a table that lives in L2.  Probing never wraps: the table
-//    has kPad slots past its capacity.  Within a warp, a run of consecutive
+//    (asc << b) | desc, b = ceil(log2 n).  There are at most B = min(n,
+//    #minima * #maxima) distinct pairs; the capacity is a power of two >= 2 B
+//    while 2 B <= n, else >= B, chosen on the device, so smooth fields (few
+//    extrema) use a table that lives in L2.  kPad slots past the capacity keep
+//    probes from wrapping (nearly always) and a slot free (always).  Within a warp, a run of consecutive
 //    vertices with the same key (neighbours usually share a cell) probes
 //    once.  Each vertex keeps its slot in `ms` for now.
 // 2. Ranks, by one of two routes chosen on the device:
@@ -26,7 +26,8 @@
 //        global sort.
 //    (b) otherwise -- small tables with random home slots, a group or a
 //        chunk too big for (a), a caller that needs the sorted keys --
-//        the occupied slots are compacted, radix-sorted by key and ranked.
+//        the occupied slots are compacted, radix-sorted by key and ranked
+//        (run_pair_ranks).
 // 3. ms[v] = table_vals[ms[v]].
 #include <cuda_runtime.h>
 
@@ -171,6 +172,7 @@ __device__ __forceinline__ uint32_t slot_base(uint32_t asc, unsigned long long f
 // far-reaching extremum spread out with their other ends.
 __device__ __forceinline__ uint32_t home_slot(uint32_t asc, uint32_t desc, uint32_t cap, unsigned long long f, bool both) {
     // 32-bit hashes: a 64-bit finaliser was a quarter of the insert's instructions
+    // (multipliers: primes of xxHash32)
     const uint32_t hd = desc * 0x9E3779B1u;
     if (cap <= kCacheResidentSlots) {  // fits in cache: spread
         uint32_t h = (hd ^ asc) * 0x85EBCA77u;

@@ -16,7 +16,8 @@
 //               super-tile's first output position for that digit;
 //   k_ord_down  each block takes super-tiles s, s + G, s + 2G, ... (G
 //               blocks), walks their tiles in order, ranks each tile's keys
-//               stably (warp ballots), keeps running per-digit offsets and
+//               stably (the lanes of a digit meet in a word of shared memory,
+//               or by match where few digits occur), keeps running per-digit offsets and
 //               writes through shared memory in coalesced runs.  The next
 //               tile is fetched by a 1D TMA bulk copy into the other half
 //               of a shared-memory double buffer while the current one is
@@ -26,7 +27,7 @@
 //               completed in L2 before they are written back.
 // The last pass files (vertex id, position) pairs into buckets of
 // consecutive ids instead of writing sorted keys, and the order field is
-// their inverse permutation (k_pair_permute); while the
+// their inverse permutation (k_ord_permute); while the
 // order array fits the L2 it scatters the positions itself.  Small fields go
 // through all four passes in one cooperative launch (k_ord_coop).
 #include <cuda_runtime.h>
@@ -283,13 +284,13 @@ struct DownArgs {
 constexpr size_t kBufWords = 2 * kTile;
 constexpr size_t kDownSmem = 2 * kBufWords * 4 + kW * kB * 2 + 2 * kB * 4 + 32 * 4 + 2 * kB * 4 + 2 * 8 + kW * kB * 4;
 
-// Lanes of the warp holding the same digit as this lane: one match
-// instruction, whose cost grows with the number of distinct digits in the
-// warp, or a word of shared memory per digit (rank_in_warp), which a few
-// digits would crowd.  The middle passes of a 512^3 field took 1.62 ms with
-// eight ballots per key (issue-bound) and take 1.39 this way (LSU 79 %, DRAM
-// half busy); shares of the keys by ballots were no faster (1.41 to 1.5).
-
+// The downsweep.  A key's rank among the warp's lanes with its digit comes
+// from one match instruction, whose cost grows with the number of distinct
+// digits in the warp, or from a word of shared memory per digit
+// (rank_in_warp), which a few digits would crowd.  The middle passes of a 512^3
+// field took 1.62 ms with eight ballots per key (issue-bound) and take 1.39 this
+// way (LSU 79 %, DRAM half busy); shares of the keys by ballots were no faster
+// (1.41 to 1.5).
 template <int OUT, int SHIFT>
 __global__ void __launch_bounds__(kT, MSC_ORD_MIN_BLOCKS) k_ord_down(const DownArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];

@@ -1,8 +1,7 @@
 // Onesweep LSD radix sorts: the vertex order of many packed instances at
 // once (Simulation of Simplicity, section "Preprocessing": sort by value,
-// ties by global id, per instance) and 64-bit keys with an int32 payload
-// (unique Morse-Smale pairs, region-adjacency keys); plus the inversion of
-// the vertex order that order.cu shares.
+// ties by global id, per instance), 64-bit keys with or without an int32
+// payload (region adjacency), and the ranks of the distinct Morse-Smale pairs.
 //
 // Keys of a float field: float32 bits mapped to an order-preserving uint32
 // (-0.0 first folded onto +0.0 so that the two tie, as IEEE '<' says).
@@ -10,10 +9,11 @@
 // the first pass reads the vertices in id order, so equal keys stay in id
 // order: the final position of v is its rank under (f[v], v).
 //
-// One pass = one kernel.  A block takes tiles of 4096 keys from a global
+// One pass = one kernel (the pair ranks make all of theirs in one).  A block
+// takes tiles of 4096 keys (64-bit ones: 6144) from a global
 // atomic counter (so every predecessor tile is owned by a running block),
-// ranks its keys per digit stably within each warp (ballot peers +
-// per-warp counters), publishes its per-digit counts to a decoupled
+// ranks its keys per digit stably within each warp (the lanes of a digit meet
+// in a word of shared memory), publishes its per-digit counts to a decoupled
 // look-back array, sums its predecessors' counts and scatters through
 // shared memory.  The last pass of an order files (vertex id, position)
 // pairs into buckets of consecutive ids; the order field is their inverse

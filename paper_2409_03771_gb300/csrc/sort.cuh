@@ -1,5 +1,5 @@
-// Onesweep LSD radix sort: float32 -> vertex order, and 64-bit keys with an
-// int32 payload (used to sort unique Morse-Smale pairs).
+// Radix sorts: float32 -> vertex order (one field, packed fields), 64-bit keys
+// with or without an int32 payload, and the ranks of a hash table's keys.
 #pragma once
 
 #include "common.cuh"

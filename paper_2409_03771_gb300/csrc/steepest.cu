@@ -346,7 +346,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_steepest_ld(const int32_t* __re
 // are packed ids (instance offset + local id).  ext[2i], ext[2i+1] count
 // the instance's minima and maxima.  96 grids, 45M vertices: 437 us with a
 // division per cell of the box and a search and a barrier per tile, 351 now
-// (three blocks per SM; four spill, 370).
+// (three blocks per SM; four spill, 370).  At three the 16-wide shapes spill 16
+// bytes and the 64-bit variants up to 120, and are still the faster ones: 96
+// grids of noise 619, 648, 682, 666 us by shape before, 492, 579, 461, 584 now; one
+// of 517^3 (64-bit) 2050 to 2159, 1576 to 1732 now.
 
 constexpr int kSmemTileTable = 2048;  // instances whose tile table goes to shared memory
 
