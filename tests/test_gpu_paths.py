@@ -373,29 +373,36 @@ def test_cc_mask_small_grids(m, oracle_mod, conn, dims, density, offset):
     np.testing.assert_array_equal(host(lab), oracle_mod.cc_grid(mask, dims, conn))
 
 
-# (mask, 6 or 14 neighbours, stage, us per call): between what the stage takes and what it took with finds one after
-# the other and run starts from masks (1550, 2270 and 104 us) or in chunks of 8192 voxels (14 us)
-@pytest.mark.parametrize("dims,kind,conn,stage,limit", [((512, 512, 512), 0.5, 6, "cc.local", 1300.0),
-                                                        ((512, 512, 512), 0.5, 14, "cc.local", 1900.0),
-                                                        ((203, 150, 177), "checker", 14, "cc.merge", 85.0),
-                                                        ((48, 48, 48), 0.5, 6, "cc.flatten", 10.0)])
-def test_cc_mask_stage_times(m, dims, kind, conn, stage, limit):
+def traced(m, call, reps=6):
+    """Best device time of each stage over a few calls, ms."""
+    call()
+    best = {}
+    for _ in range(reps):
+        m.msc_trace_reset()
+        m.msc_trace_enable(True)
+        call()
+        m.msc_trace_enable(False)
+        for k, v in m.msc_trace_collect().items():
+            best[k] = min(best.get(k, v[1]), v[1])
+    m.msc_trace_reset()
+    return best
+
+
+# a stage's time against another's on the same GPU: between the ratio now and the one with finds one after the other
+# and run starts from masks (5.9, 8.3), contacts past the queue united lane by lane (0.78), chunks of 8192 voxels (0.5)
+@pytest.mark.parametrize("dims,kind,conn,stage,against,limit", [
+    ((512, 512, 512), 0.5, 6, "cc.local", "full", 5.0), ((512, 512, 512), 0.5, 14, "cc.local", "full", 7.1),
+    ((203, 150, 177), "checker", 14, "cc.merge", "cc.local", 0.65), ((48, 48, 48), 0.5, 6, "cc.flatten", "cc.local", 0.35)])
+def test_cc_mask_stage_times(m, dims, kind, conn, stage, against, limit):
     n = dims[0] * dims[1] * dims[2]
     if kind == "checker":
         i = torch.arange(n, device="cuda")
         mask = ((i % dims[0] + i // dims[0] % dims[1] + i // (dims[0] * dims[1])) & 1).to(torch.uint8)
     else:
         mask = (torch.rand(n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1)) < kind).to(torch.uint8)
-    times = []
-    m.cc_mask(mask, dims, conn)
-    for _ in range(6):
-        m.msc_trace_reset()
-        m.msc_trace_enable(True)
-        m.cc_mask(mask, dims, conn)
-        m.msc_trace_enable(False)
-        times.append(m.msc_trace_collect()[stage][1] * 1e3)
-    m.msc_trace_reset()
-    assert min(times) < limit, times
+    t = traced(m, lambda: m.cc_mask(mask, dims, conn))
+    ref = t if against != "full" else traced(m, lambda: m.cc_mask(torch.ones_like(mask), dims, conn))
+    assert t[stage] < limit * ref[against if against != "full" else stage], (t, ref)
 
 
 # ---------------------------------------------------------------------------
@@ -451,17 +458,10 @@ def test_batch_of_noise_with_many_pairs(m, dims):
             assert torch.equal(got[lo:hi], want)
 
 
-def test_pair_ranks_time_per_pair(m):
-    """Tens of millions of pairs: 0.09 us per thousand with onesweep passes (0.086 as launches), 0.125 without."""
+def test_pair_ranks_time_of_many_pairs(m):
+    """A third as many pairs as vertices: against the middle passes of the batched order twice as long with onesweep
+    passes, three times with the passes for few pairs."""
     b = m.Batch([(400, 400, 400)])
     b.f.copy_(torch.rand(b.total, device="cuda", generator=torch.Generator(device="cuda").manual_seed(3)))
-    b.run()
-    times = []
-    for _ in range(4):
-        m.msc_trace_reset()
-        m.msc_trace_enable(True)
-        b.run()
-        m.msc_trace_enable(False)
-        times.append(m.msc_trace_collect()["msid.pairs"][1] * 1e6)
-    m.msc_trace_reset()
-    assert min(times) / int(b.num_cells[0]) < 0.108, (times, int(b.num_cells[0]))
+    t = traced(m, b.run, 4)
+    assert t["msid.pairs"] < 2.5 * t["order.pass"], t
